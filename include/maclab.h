@@ -149,7 +149,7 @@ typedef struct {
     int64_t n_fast;          /* nodes updated on the interior fast path        */
     size_t device_bytes;     /* device memory held by the handle               */
     int tile_rows;           /* rows per warp strip of the strip kernel        */
-    int step_kernel;         /* maclab_step_kernel in use                      */
+    int step_kernel;         /* maclab_step_kernel of single-step launches     */
     int dirichlet_fused;     /* 1 when Dirichlet nodes are set inside the step kernel */
     int temporal_block;      /* steps per launch of interior tiles: 1 or 2     */
     int64_t clean_tiles;     /* tiles that can take two steps per launch (0 until
@@ -183,9 +183,12 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
 /* Change the stream later calls launch on (cudaStream_t). */
 int maclab_set_stream(maclab_t sim, void* stream);
 
-/* Advance n >= 0 steps (procedure steps (c)-(e) of Section 3): one launch
- * of the fused step kernel per step, plus the Dirichlet kernel when the grid
- * has Dirichlet nodes.  Asynchronous on the handle's stream. */
+/* Advance n >= 0 steps (procedure steps (c)-(e) of Section 3): on small
+ * grids several steps per launch (each block steps a tile with a halo of
+ * several nodes in shared memory), otherwise one launch of the fused step
+ * kernel per step, plus the Dirichlet kernel when the grid has Dirichlet
+ * nodes it does not handle itself.  Results are bitwise identical either
+ * way.  Asynchronous on the handle's stream. */
 int maclab_step(maclab_t sim, int64_t n);
 
 /* Steps per CUDA-graph replay in maclab_step (an even number, 0 = off;
@@ -301,7 +304,8 @@ int maclab_set_launch(maclab_t sim, int rows, int blocks);
 
 /* Choose the step kernel (maclab_step_kernel).  MACLAB_KERNEL_TMA needs an
  * FP32 handle; otherwise MACLAB_E_ARG.  Tuning only: results are bitwise
- * identical.  A TMA-staged step whose copy never arrives (a wait bounded
+ * identical.  From then on every step is a launch of that kernel (no
+ * several-step launches on small grids).  A TMA-staged step whose copy never arrives (a wait bounded
  * at about a second) makes the next maclab_residual / maclab_get_state
  * return MACLAB_E_CUDA. */
 int maclab_set_step_kernel(maclab_t sim, int kernel);
@@ -365,7 +369,9 @@ int maclab_get_profile(maclab_t sim, double* step_kernel_ms, int64_t* launches);
  * on clean tiles (maclab_set_temporal_block(sim, 2)), 7 for the row-march
  * kernel, 8 for the row-march kernel with two steps per pass on plain strip
  * blocks; 5, 6 and 8 are tried on FP32 MacLABSWE handles only, and the
- * temporal block depth is set to the winner's (1 unless 6 or 8 wins).  Each shape runs 2 + trial_steps steps; the
+ * temporal block depth is set to the winner's (1 unless 6 or 8 wins).  On a
+ * small grid the several-step launches of maclab_step are timed too and kept
+ * on when they beat every shape.  Each shape runs 2 + trial_steps steps; the
  * state, step count and time are restored afterwards (results are bitwise
  * identical for every shape).  Allocates and frees a copy of the state.
  * Synchronises. */

@@ -18,8 +18,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libmaclab.so")
-SOURCES = [os.path.join(CSRC, "maclab.cu"), os.path.join(CSRC, "warmstart.cu")]
-DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")] + \
+SOURCES = [os.path.join(CSRC, f) for f in ("maclab.cu", "window.cu", "warmstart.cu")]
+DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))] + \
     [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE) if f.endswith(".h")]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

@@ -10,6 +10,7 @@
 #include "maclab_kernels.cuh"
 #include "maclab_march.cuh"
 #include "maclab_elab.cuh"
+#include "window.h"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -111,6 +112,12 @@ struct maclab_s {
     void* gdist[2] = {nullptr, nullptr};  // 9 planes of [ny][pitch] per buffer
     void* snap[3] = {nullptr, nullptr, nullptr};  // marked state (eta, u, v), allocated on first mark
     int64_t mark_n = -1;       // step count of the marked state (-1: none)
+    // several steps per launch (small grids; maclab_window.cuh)
+    bool kernel_chosen = false;    // the caller picked a step kernel: every step is a launch of it
+    window::Plan wplan;            // k = 0: not used on this grid
+    window::Item* witems = nullptr;
+    void* winst = nullptr;         // BatchInst<T>[1]
+    void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches
     std::vector<cudaEvent_t> events;  // pairs around step-kernel launches
     size_t events_used = 0;
     std::string err;
@@ -476,9 +483,86 @@ int launch_pair(maclab_t s)
     return MACLAB_OK;
 }
 
+bool use_window(const maclab_s* s)
+{
+    return s->wplan.k > 0 && !s->kernel_chosen && s->tblock == 1 && !s->elab && !s->newlevel;
+}
+
+// Steps of each of the launches that take n steps at most k at a time: one
+// launch for a single step, two or more otherwise (the last of them reads
+// the scratch state, so that it can leave the last two states in the
+// handle's two buffers, where the residual looks for them).
+struct WindowRun {
+    int64_t launches, base, more;
+    WindowRun(int64_t n, int k) : launches(std::max<int64_t>(n > 1 ? 2 : 1, (n + k - 1) / k)), base(n / launches), more(n % launches) {}
+    int steps(int64_t i) const { return (int)(base + (i < more ? 1 : 0)); }
+    bool to_scratch(int64_t i) const { return (launches - 2 - i) % 2 == 0; }  // i < launches - 1
+};
+
+// State buffers of launch i: cur -> other for a single step; otherwise
+// cur -> scratch / other in turn, ending scratch -> cur with the state
+// before the last step in other.
+template <typename T>
+window::Buffers<T> window_buffers(const WindowRun& r, int64_t i, void* const (&eta)[2], void* const (&u)[2],
+                                  void* const (&v)[2], void* const (&mid)[3], int cur)
+{
+    void* A[3] = {eta[cur], u[cur], v[cur]};
+    void* B[3] = {eta[1 - cur], u[1 - cur], v[1 - cur]};
+    window::Buffers<T> b{};
+    for (int q = 0; q < 3; ++q) {
+        b.in[q] = (const T*)(i == 0 ? A[q] : r.to_scratch(i - 1) ? mid[q] : B[q]);
+        if (r.launches == 1) {
+            b.out[q] = (T*)B[q];
+        } else if (i < r.launches - 1) {
+            b.out[q] = (T*)(r.to_scratch(i) ? mid[q] : B[q]);
+        } else {
+            b.out[q] = (T*)A[q];
+            b.prev[q] = (T*)B[q];
+        }
+    }
+    return b;
+}
+
+template <typename T>
+int advance_window(maclab_t s, int64_t n)
+{
+    const WindowRun r(n, s->wplan.k);
+    for (int64_t i = 0; i < r.launches; ++i) {
+        const int steps = r.steps(i);
+        cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+        if (s->profiling) {
+            while (s->events.size() < s->events_used + 2) {
+                cudaEvent_t ev;
+                if (cudaEventCreate(&ev) != cudaSuccess) return cuda_fail(s, cudaGetLastError(), "event");
+                s->events.push_back(ev);
+            }
+            ev0 = s->events[s->events_used];
+            ev1 = s->events[s->events_used + 1];
+            s->events_used += 2;
+            s->prof_steps += steps;
+            cudaEventRecord(ev0, s->stream);
+        }
+        window::DirTable tab;
+        const bool steady = s->steady_bc || s->n_dir == 0;
+        if (!steady)
+            for (int k = 0; k < steps; ++k) tab.v[k] = dir_values(s, s->n + k + 1);
+        const cudaError_t e = window::launch<T>(s->wplan, s->winst, s->witems, nullptr,
+                                                window_buffers<T>(r, i, s->eta, s->u, s->v, s->wmid, s->cur), steps,
+                                                steady ? nullptr : &tab, s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "step launch");
+        if (s->profiling) cudaEventRecord(ev1, s->stream);
+        s->n += steps;
+    }
+    if (r.launches == 1) s->cur = 1 - s->cur;
+    s->have_prev = true;
+    return MACLAB_OK;
+}
+
 // n steps: pairs where temporal blocking is on, the last step always single
 int advance(maclab_t s, int64_t n)
 {
+    if (n > 0 && use_window(s))
+        return s->prec == MACLAB_F32 ? advance_window<float>(s, n) : advance_window<double>(s, n);
     const bool pairs_on = s->tblock == 2 && s->prec == MACLAB_F32 && !s->elab && !s->newlevel;
     const int64_t pairs = pairs_on && n >= 3 ? (n - 1) / 2 : 0;
     for (int64_t k = 0; k < pairs; ++k) {
@@ -969,6 +1053,65 @@ int setup_march(maclab_t s, const Prepared& P, int sms)
     return MACLAB_OK;
 }
 
+// Fields of one grid in a packed buffer set, for both buffer parities.
+template <typename T>
+BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u)[2], void* const (&v)[2], void* D,
+                       double* D64, uint8_t* type, size_t o)
+{
+    BatchInst<T> in{};
+    for (int par = 0; par < 2; ++par) {
+        Fields<T>& f = in.f[par];
+        f.eta = (const T*)eta[par] + o;
+        f.u = (const T*)u[par] + o;
+        f.v = (const T*)v[par] + o;
+        f.eta1 = (T*)eta[1 - par] + o;
+        f.u1 = (T*)u[1 - par] + o;
+        f.v1 = (T*)v[1 - par] + o;
+        f.D = (const T*)D + o;
+        f.type = type + o;
+        f.nx = P.nx;
+        f.ny = P.ny;
+        f.pitch = P.pitch;
+        f.idx32 = (int64_t)P.pitch * P.ny < ((int64_t)1 << 31) ? 1 : 0;
+        for (int k = 0; k < 4; ++k) f.edge[k] = P.bc.edge[k];
+        f.c = make_coef<T>(P.params, P.e, P.dt);
+    }
+    in.tiles_x = P.tiles_x;
+    in.ntiles = P.tiles_x * P.tiles_y;
+    in.D64 = D64 + o;
+    for (int k = 0; k < 4; ++k) {  // steady boundary data
+        in.bv.h[k] = P.bc.h[k].mean;
+        in.bv.qx[k] = P.bc.qx[k].mean;
+        in.bv.qy[k] = P.bc.qy[k].mean;
+    }
+    return in;
+}
+
+// Several steps per launch, where the planner finds it the better choice.
+int setup_window(maclab_t s, const Prepared& P, int sms)
+{
+    const bool f64 = s->prec == MACLAB_F64;
+    s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0}}, f64, s->fmode, sms);
+    if (s->wplan.k == 0) return MACLAB_OK;
+    const size_t NP = (size_t)P.pitch * P.ny, items = s->wplan.items.size() * sizeof(window::Item);
+    bool ok = (s->witems = (window::Item*)dev_alloc(s, items)) != nullptr &&
+              (s->winst = dev_alloc(s, f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>))) != nullptr;
+    for (int q = 0; q < 3 && ok; ++q) ok = (s->wmid[q] = dev_alloc(s, NP * s->esize)) != nullptr;
+    if (!ok) return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
+    cudaError_t e = cudaMemcpyAsync(s->witems, s->wplan.items.data(), items, cudaMemcpyHostToDevice, s->stream);
+    BatchInst<float> f{};
+    BatchInst<double> d{};
+    if (f64) d = make_inst<double>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, 0);
+    else f = make_inst<float>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, 0);
+    if (e == cudaSuccess)
+        e = f64 ? cudaMemcpyAsync(s->winst, &d, sizeof(d), cudaMemcpyHostToDevice, s->stream)
+                : cudaMemcpyAsync(s->winst, &f, sizeof(f), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = window::prepare_launch(s->wplan, f64);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "upload");
+    return MACLAB_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1164,7 +1307,8 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
     s->ty = choose_tile_rows(ny, s->ncb, sms);
     s->nrb = (ny + s->ty - 1) / s->ty;
     {
-        const int mrc = setup_march(s, P, sms);
+        int mrc = setup_march(s, P, sms);
+        if (mrc == MACLAB_OK) mrc = setup_window(s, P, sms);
         if (mrc != MACLAB_OK) {
             release_all(s);
             delete s;
@@ -1288,7 +1432,8 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
     const int cur = s->cur;
     const int64_t n0 = s->n;
     const bool hp = s->have_prev;
-    const int kernel0 = s->kernel;
+    const bool chosen0 = s->kernel_chosen;
+    s->kernel_chosen = true;  // time the launch shapes themselves
     const int ty0 = s->ty;
     const int prof0 = s->profiling;
     // candidates: 0 = tile kernel; k = 1..4 strip kernel with 4 << k rows;
@@ -1342,19 +1487,35 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
             best_k = k;
         }
     }
+    // several steps per launch, kept on when it beats every shape
+    bool keep_window = false;
+    if (rc == MACLAB_OK && s->wplan.k > 0) {
+        s->tblock = 1;
+        s->kernel_chosen = false;
+        if (use_window(s)) {
+            rc = maclab_step(s, 2);
+            cudaEventRecord(e0, s->stream);
+            if (rc == MACLAB_OK) rc = maclab_step(s, trial_steps);
+            cudaEventRecord(e1, s->stream);
+            cudaEventSynchronize(e1);
+            float ms = 0;
+            cudaEventElapsedTime(&ms, e0, e1);
+            keep_window = rc == MACLAB_OK && ms < best;
+        }
+    }
+    s->kernel_chosen = rc == MACLAB_OK ? !keep_window : chosen0;
     s->events_used = 0;
     s->profiling = prof0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     s->kernel = kernel_of_choice(best_k);
-    s->tblock = best_k == 6 || best_k == 8 ? 2 : 1;
+    s->tblock = !keep_window && (best_k == 6 || best_k == 8) ? 2 : 1;
     if (best_k >= 1 && best_k <= 4) {
         s->ty = std::min(rows[best_k], s->grid.ny);
     } else {
         s->ty = ty0;
     }
     s->nrb = (s->grid.ny + s->ty - 1) / s->ty;
-    (void)kernel0;
     drop_graphs(s);
     for (int k = 0; k < 6; ++k) cudaMemcpyAsync(src[k], keep[k], bytes, cudaMemcpyDeviceToDevice, s->stream);
     cudaStreamSynchronize(s->stream);
@@ -1633,6 +1794,7 @@ int maclab_set_step_kernel(maclab_t s, int kernel)
     if (kernel == MACLAB_KERNEL_TMA && !s->tma_ok)
         return fail(s, MACLAB_E_ARG, "the TMA-staged kernel needs an FP32 handle with 16-byte aligned buffers");
     s->kernel = kernel;
+    s->kernel_chosen = true;
     drop_graphs(s);
     return MACLAB_OK;
 }
@@ -2014,6 +2176,9 @@ struct maclab_batch_s {
     unsigned int bar_polls = BARRIER_POLLS;  // polls before a grid-barrier wait gives up
     bool broken = false;            // a persistent step stopped early: the state must be reloaded
     std::vector<uint8_t> reloaded;  // instances set since the batch broke
+    window::Plan wplan;             // several steps per launch (k = 0: not used)
+    window::Item* witems = nullptr;
+    void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches, packed
     void* snap[3] = {nullptr, nullptr, nullptr};  // marked state, packed like eta / u / v
     int64_t mark_n = -1;            // step count of the marked state (-1: none)
     std::string err;
@@ -2064,35 +2229,8 @@ void fill_insts(maclab_batch_t b, const std::vector<Prepared>& P, std::vector<Ba
 {
     out.resize(b->count);
     for (int i = 0; i < b->count; ++i) {
-        BatchInst<T>& in = out[i];
-        const size_t o = b->off[i];
-        for (int par = 0; par < 2; ++par) {
-            Fields<T>& f = in.f[par];
-            f.eta = (const T*)b->eta[par] + o;
-            f.u = (const T*)b->u[par] + o;
-            f.v = (const T*)b->v[par] + o;
-            f.eta1 = (T*)b->eta[1 - par] + o;
-            f.u1 = (T*)b->u[1 - par] + o;
-            f.v1 = (T*)b->v[1 - par] + o;
-            f.D = (const T*)b->D + o;
-            f.type = b->type + o;
-            f.nx = P[i].nx;
-            f.ny = P[i].ny;
-            f.pitch = P[i].pitch;
-            f.idx32 = (int64_t)P[i].pitch * P[i].ny < ((int64_t)1 << 31) ? 1 : 0;
-            for (int k = 0; k < 4; ++k) f.edge[k] = P[i].bc.edge[k];
-            f.c = make_coef<T>(P[i].params, P[i].e, P[i].dt);
-        }
-        in.tiles_x = P[i].tiles_x;
-        in.tile0 = b->tile0[i];
-        in.ntiles = b->ntiles[i];
-        in.pad = 0;
-        in.D64 = b->D64 + o;
-        for (int k = 0; k < 4; ++k) {  // steady boundary data
-            in.bv.h[k] = P[i].bc.h[k].mean;
-            in.bv.qx[k] = P[i].bc.qx[k].mean;
-            in.bv.qy[k] = P[i].bc.qy[k].mean;
-        }
+        out[i] = make_inst<T>(P[i], b->eta, b->u, b->v, b->D, b->D64, b->type, b->off[i]);
+        out[i].tile0 = b->tile0[i];
     }
 }
 
@@ -2195,9 +2333,31 @@ int batch_launch(maclab_batch_t b, cudaStream_t st)
     return MACLAB_OK;
 }
 
-int batch_one(maclab_batch_t b, cudaStream_t st)
+template <typename T>
+int batch_window(maclab_batch_t b, int64_t n, cudaStream_t st)
 {
-    return b->prec == MACLAB_F32 ? batch_launch<float>(b, st) : batch_launch<double>(b, st);
+    const WindowRun r(n, b->wplan.k);
+    for (int64_t i = 0; i < r.launches; ++i) {
+        const cudaError_t e =
+            window::launch<T>(b->wplan, b->insts, b->witems, b->active,
+                              window_buffers<T>(r, i, b->eta, b->u, b->v, b->wmid, b->cur), r.steps(i), nullptr, st);
+        if (e != cudaSuccess) return bfail(b, MACLAB_E_CUDA, std::string("batch step launch: ") + cudaGetErrorString(e));
+    }
+    if (r.launches == 1) b->cur = 1 - b->cur;
+    b->n += n;
+    b->have_prev = true;
+    return MACLAB_OK;
+}
+
+int batch_steps(maclab_batch_t b, int64_t n, cudaStream_t st)
+{
+    const bool f32 = b->prec == MACLAB_F32;
+    if (n > 0 && b->wplan.k > 0) return f32 ? batch_window<float>(b, n, st) : batch_window<double>(b, n, st);
+    for (int64_t k = 0; k < n; ++k) {
+        const int rc = f32 ? batch_launch<float>(b, st) : batch_launch<double>(b, st);
+        if (rc != MACLAB_OK) return rc;
+    }
+    return MACLAB_OK;
 }
 
 int batch_capture(maclab_batch_t b)
@@ -2212,7 +2372,7 @@ int batch_capture(maclab_batch_t b)
     int rc = MACLAB_OK;
     e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        for (int k = 0; k < b->graph_steps && rc == MACLAB_OK; ++k) rc = batch_one(b, b->capture_stream);
+        rc = batch_steps(b, b->graph_steps, b->capture_stream);
         e = cudaStreamEndCapture(b->capture_stream, &g);
     }
     b->cur = cur;
@@ -2445,6 +2605,36 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         delete b;
         return MACLAB_E_CUDA;
     }
+    {
+        std::vector<window::GridView> views;
+        int fmode = 0, dev = 0, sms = 0;
+        for (int i = 0; i < count; ++i) {
+            views.push_back(window::GridView{P[i].nx, P[i].ny, P[i].pitch, P[i].bc.edge, P[i].type.data(), (long long)b->off[i]});
+            fmode |= P[i].fmode;
+        }
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        b->wplan = window::make_plan(views, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
+        if (b->wplan.k > 0) {
+            const size_t bytes = b->wplan.items.size() * sizeof(window::Item);
+            bool got = (b->witems = (window::Item*)bdev_alloc(b, bytes)) != nullptr;
+            for (int q = 0; q < 3 && got; ++q) got = (b->wmid[q] = bdev_alloc(b, NP * b->esize)) != nullptr;
+            if (!got) {
+                brelease(b);
+                delete b;
+                return bfail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
+            }
+            ce = cudaMemcpyAsync(b->witems, b->wplan.items.data(), bytes, cudaMemcpyHostToDevice, b->stream);
+            if (ce == cudaSuccess) ce = window::prepare_launch(b->wplan, b->prec == MACLAB_F64);
+            if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
+            if (ce != cudaSuccess) {
+                bfail(nullptr, MACLAB_E_CUDA, std::string("batch upload: ") + cudaGetErrorString(ce));
+                brelease(b);
+                delete b;
+                return MACLAB_E_CUDA;
+            }
+        }
+    }
     *out = b;
     for (int i = 0; i < count; ++i) {
         if (h0 && h0[i]) {
@@ -2478,11 +2668,7 @@ int maclab_batch_step(maclab_batch_t b, int64_t n)
         b->have_prev = true;
         n -= b->graph_steps;
     }
-    for (int64_t k = 0; k < n; ++k) {
-        int rc = batch_one(b, b->stream);
-        if (rc != MACLAB_OK) return rc;
-    }
-    return MACLAB_OK;
+    return batch_steps(b, n, b->stream);
 }
 
 int maclab_batch_set_graph_steps(maclab_batch_t b, int steps)

@@ -696,16 +696,16 @@ struct NodeQ {  // per-node quantities for the general path
     T eta, D, h, u, v, uu, Fx, Fy;
 };
 
+// Node quantities of a raw state, mirrored for a specular ghost (flip).
 template <typename T>
-__device__ __forceinline__ NodeQ<T> node_q(const Fields<T>& f, size_t idx, uint8_t flip)
+__device__ __forceinline__ NodeQ<T> node_q_of(const Coef<T>& c, T eta, T D, T u, T v, uint8_t flip)
 {
     using O = Op<T>;
-    const Coef<T>& c = f.c;
     NodeQ<T> n;
-    n.eta = f.eta[idx];
-    n.D = f.D[idx];
-    n.u = f.u[idx];
-    n.v = f.v[idx];
+    n.eta = eta;
+    n.D = D;
+    n.u = u;
+    n.v = v;
     T wfx = c.wfx, wfy = c.wfy, Om = c.Om;
     if (flip & 1) { n.u = -n.u; wfx = -wfx; }
     if (flip & 2) { n.v = -n.v; wfy = -wfy; }
@@ -718,20 +718,50 @@ __device__ __forceinline__ NodeQ<T> node_q(const Fields<T>& f, size_t idx, uint8
     n.Fy = O::fma(-cbs, n.v, O::fma(-omh, n.u, wfy));
     return n;
 }
-
-// f^eq_a(h,u) - f^eq_a(D,0) for direction a != 0 with lattice vector (cx, cy)
 template <typename T>
-__device__ __forceinline__ T feq_diff(const Coef<T>& c, const NodeQ<T>& n, int cx, int cy)
+__device__ __forceinline__ NodeQ<T> node_q(const Fields<T>& f, size_t idx, uint8_t flip)
+{
+    return node_q_of(f.c, f.eta[idx], f.D[idx], f.u[idx], f.v[idx], flip);
+}
+
+// f^eq_a(h,u) - f^eq_a(D,0) for direction a != 0 with lattice vector
+// (cx, cy) and weight lambda_a = lam
+template <typename T>
+__device__ __forceinline__ T feq_diff_dir(const Coef<T>& c, const NodeQ<T>& n, T cx, T cy, T lam)
 {
     using O = Op<T>;
-    const T lam = (cx != 0 && cy != 0) ? T(0.25) : T(1);
-    const T cu = O::fma(T(cx), n.u, O::mul(T(cy), n.v));
+    const T cu = O::fma(cx, n.u, O::mul(cy, n.v));
     const T hcu = O::mul(n.h, cu);
     T acc = O::mul(O::mul(c.G6, n.eta), O::fma(T(2), n.D, n.eta));
     acc = O::fma(hcu, c.k3, acc);
     acc = O::fma(O::mul(hcu, cu), c.k2, acc);
     acc = O::fma(-c.K6, O::mul(n.h, n.uu), acc);
     return O::mul(lam, acc);
+}
+template <typename T>
+__device__ __forceinline__ T feq_diff(const Coef<T>& c, const NodeQ<T>& n, int cx, int cy)
+{
+    return feq_diff_dir(c, n, T(cx), T(cy), (cx != 0 && cy != 0) ? T(0.25) : T(1));
+}
+
+// The a = 0 term of Eq. Mac.lb.6 of a node in perturbation form (the start
+// of its eta sum), and its velocities from the momentum sums.
+template <typename T>
+__device__ __forceinline__ T general_rest(const Coef<T>& c, const NodeQ<T>& X)
+{
+    using O = Op<T>;
+    const T Sh = O::fma(-O::mul(T(5), O::mul(c.G6, X.eta)), O::fma(T(2), X.D, X.eta), X.eta);
+    return O::fma(-O::mul(T(4), c.K6), O::mul(X.h, X.uu), Sh);
+}
+template <typename T>
+__device__ __forceinline__ void general_finish(const Coef<T>& c, const NodeQ<T>& X, T Sh, T Sx, T Sy, bool noslip,
+                                               T& u1, T& v1)
+{
+    using O = Op<T>;
+    const T hu1 = O::mul(c.e, Sx), hv1 = O::mul(c.e, Sy);
+    const T inv = T(1) / O::add(X.D, Sh);
+    u1 = noslip ? T(0) : O::mul(hu1, inv);
+    v1 = noslip ? T(0) : O::mul(hv1, inv);
 }
 
 // Update of one node (i, j) with the links resolved one by one.  Every
@@ -746,8 +776,7 @@ __device__ __forceinline__ void general_node(const Fields<T>& f, int i, int j)
     const size_t xi = (size_t)j * f.pitch + i;
     const Coef<T>& c = f.c;
     const NodeQ<T> X = node_q(f, xi, 0);
-    T Sh = O::fma(-O::mul(T(5), O::mul(c.G6, X.eta)), O::fma(T(2), X.D, X.eta), X.eta);
-    Sh = O::fma(-O::mul(T(4), c.K6), O::mul(X.h, X.uu), Sh);
+    T Sh = general_rest(c, X);
     T Sx = T(0), Sy = T(0);
     T Q = T(0), Qx = T(0), Qy = T(0);  // new level: sum of lambda G6 (D_x - D_y), weighted by 1, c_x, c_y
 #pragma unroll 1
@@ -791,10 +820,8 @@ __device__ __forceinline__ void general_node(const Fields<T>& f, int i, int j)
         Sx = O::fma(Sh, Qx, Sx);
         Sy = O::fma(Sh, Qy, Sy);
     }
-    const T hu1 = O::mul(c.e, Sx), hv1 = O::mul(c.e, Sy);
-    const T inv = T(1) / O::add(X.D, Sh);
-    T u1 = O::mul(hu1, inv), v1 = O::mul(hv1, inv);
-    if ((f.type[xi] & KIND_MASK) == K_NOSLIP) { u1 = T(0); v1 = T(0); }
+    T u1, v1;
+    general_finish(c, X, Sh, Sx, Sy, (f.type[xi] & KIND_MASK) == K_NOSLIP, u1, v1);
     f.eta1[xi] = Sh;
     f.u1[xi] = u1;
     f.v1[xi] = v1;
@@ -822,21 +849,29 @@ struct DirValues {
     double h[4], qx[4], qy[4];  // prescribed values at t_{n+1} per edge
 };
 
+// Node x with inward node n1 in arrays eta, u, v, D; D64: the node's own
+// still-water depth in double.
+template <typename T>
+__device__ __forceinline__ void dirichlet_value(T* eta, T* u, T* v, const T* D, double D64, int x, int n1, int meta,
+                                                const DirValues& bv)
+{
+    const int kind = meta & 15, ed = meta >> 4;
+    if (kind == K_DIR_H) {
+        eta[x] = (T)(bv.h[ed] - D64);
+        u[x] = u[n1];
+        v[x] = v[n1];
+        return;
+    }
+    const double h = kind == K_DIR_Q ? (double)D[n1] + (double)eta[n1] : bv.h[ed];
+    eta[x] = (T)(h - D64);
+    u[x] = (T)(bv.qx[ed] / h);
+    v[x] = (T)(bv.qy[ed] / h);
+}
 template <typename T>
 __device__ __forceinline__ void dirichlet_node(T* eta, T* u, T* v, const T* D, const double* D64, const DirNode d,
                                                const DirValues& bv)
 {
-    const int kind = d.meta & 15, ed = d.meta >> 4;
-    if (kind == K_DIR_H) {
-        eta[d.x] = (T)(bv.h[ed] - D64[d.x]);
-        u[d.x] = u[d.n1];
-        v[d.x] = v[d.n1];
-        return;
-    }
-    const double h = kind == K_DIR_Q ? (double)D[d.n1] + (double)eta[d.n1] : bv.h[ed];
-    eta[d.x] = (T)(h - D64[d.x]);
-    u[d.x] = (T)(bv.qx[ed] / h);
-    v[d.x] = (T)(bv.qy[ed] / h);
+    dirichlet_value(eta, u, v, D, D64[d.x], d.x, d.n1, d.meta, bv);
 }
 
 template <typename T>
@@ -1834,7 +1869,7 @@ residual_partial_kernel(const T* __restrict__ e0, const T* __restrict__ u0, cons
     }
 }
 
-__global__ void residual_final_kernel(const double* __restrict__ partial, int nblocks,
+static __global__ void residual_final_kernel(const double* __restrict__ partial, int nblocks,
                                       double* __restrict__ out)
 {
     // one warp per value, fixed order -> deterministic
