@@ -59,6 +59,7 @@ struct maclab_s {
     void* v[2] = {nullptr, nullptr};
     void* D = nullptr;         // still-water depth in the state precision
     double* D64 = nullptr;     // still-water depth in double
+    double* bed = nullptr;     // FP64: stencils of D, three planes
     uint8_t* type = nullptr;
     int* general = nullptr;    // node indices (j * nx + i) of general-link nodes
     int n_general = 0;
@@ -190,6 +191,14 @@ Coef<T> make_coef(const maclab_params& p, double e, double dt)
     c.Cb = (T)p.Cb;
     c.Om = (T)p.Omega;
     c.nz = (T)-0.0;
+    const double fs = 0.5 * e * dt;
+    c.gh = (T)(0.5 * p.g);
+    c.i3e2 = (T)(1.0 / (3.0 * e * e));
+    c.i3e = (T)(1.0 / (3.0 * e));
+    c.fwx = (T)(fs * (p.rho_a * p.Cw * p.wind_u * wmag / p.rho_w));
+    c.fwy = (T)(fs * (p.rho_a * p.Cw * p.wind_v * wmag / p.rho_w));
+    c.fCb = (T)(fs * p.Cb);
+    c.fOm = (T)(fs * p.Omega);
     return c;
 }
 
@@ -212,6 +221,8 @@ Fields<T> make_fields(const maclab_s* s)
     f.idx32 = (int64_t)s->pitch * s->grid.ny < ((int64_t)1 << 31) ? 1 : 0;
     for (int k = 0; k < 4; ++k) f.edge[k] = s->bc.edge[k];
     f.c = make_coef<T>(s->params, s->e, s->dt);
+    f.bed = (const T*)s->bed;
+    f.bed_plane = (size_t)s->pitch * s->grid.ny;
     return f;
 }
 
@@ -1056,7 +1067,7 @@ int setup_march(maclab_t s, const Prepared& P, int sms)
 // Fields of one grid in a packed buffer set, for both buffer parities.
 template <typename T>
 BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u)[2], void* const (&v)[2], void* D,
-                       double* D64, uint8_t* type, size_t o)
+                       double* D64, uint8_t* type, const double* bed, size_t plane, size_t o)
 {
     BatchInst<T> in{};
     for (int par = 0; par < 2; ++par) {
@@ -1075,6 +1086,8 @@ BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u
         f.idx32 = (int64_t)P.pitch * P.ny < ((int64_t)1 << 31) ? 1 : 0;
         for (int k = 0; k < 4; ++k) f.edge[k] = P.bc.edge[k];
         f.c = make_coef<T>(P.params, P.e, P.dt);
+        f.bed = bed ? (const T*)bed + o : nullptr;
+        f.bed_plane = plane;
     }
     in.tiles_x = P.tiles_x;
     in.ntiles = P.tiles_x * P.tiles_y;
@@ -1101,8 +1114,8 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     cudaError_t e = cudaMemcpyAsync(s->witems, s->wplan.items.data(), items, cudaMemcpyHostToDevice, s->stream);
     BatchInst<float> f{};
     BatchInst<double> d{};
-    if (f64) d = make_inst<double>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, 0);
-    else f = make_inst<float>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, 0);
+    if (f64) d = make_inst<double>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, s->bed, NP, 0);
+    else f = make_inst<float>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, nullptr, NP, 0);
     if (e == cudaSuccess)
         e = f64 ? cudaMemcpyAsync(s->winst, &d, sizeof(d), cudaMemcpyHostToDevice, s->stream)
                 : cudaMemcpyAsync(s->winst, &f, sizeof(f), cudaMemcpyHostToDevice, s->stream);
@@ -1192,6 +1205,7 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
          (s->type = (uint8_t*)dev_alloc(s, NP + 64)) && (s->stage = (double*)dev_alloc(s, 3 * N * 8)) &&
          (s->partial = (double*)dev_alloc(s, (size_t)s->red_blocks * RED_NVAL * 8)) &&
          (s->red_out = (double*)dev_alloc(s, RED_NVAL * 8));
+    if (ok && s->prec == MACLAB_F64) ok = (s->bed = (double*)dev_alloc(s, 3 * NP * 8)) != nullptr;
     if (ok && s->prec == MACLAB_F32) ok = (s->tma_err = (int*)dev_alloc(s, sizeof(int))) != nullptr;
     if (ok && !general.empty())
         ok = (s->general = (int*)dev_alloc(s, general.size() * sizeof(int))) &&
@@ -1231,6 +1245,10 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
     }
     if (!dirs.empty()) put(s->dir, dirs.data(), dirs.size() * sizeof(DirNode));
     if (s->dir_fused) put(s->dir_tile_start, dir_start.data(), dir_start.size() * sizeof(int));
+    if (s->bed && ce == cudaSuccess) {
+        bed_stencil_kernel<<<grid_blocks(N, 256, 4096), 256, 0, s->stream>>>(make_fields<double>(s), s->bed, NP);
+        ce = cudaGetLastError();
+    }
     if (s->tma_err && ce == cudaSuccess) ce = cudaMemsetAsync(s->tma_err, 0, sizeof(int), s->stream);
     for (int k = 0; k < 2 && ce == cudaSuccess; ++k) {
         ce = cudaMemsetAsync(s->eta[k], 0, NP * s->esize, s->stream);
@@ -2144,6 +2162,7 @@ struct maclab_batch_s {
     void* v[2] = {nullptr, nullptr};
     void* D = nullptr;
     double* D64 = nullptr;
+    double* bed = nullptr;          // FP64: stencils of D, three packed planes
     uint8_t* type = nullptr;
     double* stage = nullptr;
     void* insts = nullptr;          // BatchInst<T>[count]
@@ -2229,7 +2248,7 @@ void fill_insts(maclab_batch_t b, const std::vector<Prepared>& P, std::vector<Ba
 {
     out.resize(b->count);
     for (int i = 0; i < b->count; ++i) {
-        out[i] = make_inst<T>(P[i], b->eta, b->u, b->v, b->D, b->D64, b->type, b->off[i]);
+        out[i] = make_inst<T>(P[i], b->eta, b->u, b->v, b->D, b->D64, b->type, b->bed, b->total_np, b->off[i]);
         out[i].tile0 = b->tile0[i];
     }
 }
@@ -2529,6 +2548,7 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
          (b->red_out = (double*)bdev_alloc(b, (size_t)count * RED_NVAL * 8)) &&
          (b->barrier = (GridBarrier*)bdev_alloc(b, sizeof(GridBarrier))) &&
          (b->persist_err = (int*)bdev_alloc(b, sizeof(int)));
+    if (ok && b->prec == MACLAB_F64) ok = (b->bed = (double*)bdev_alloc(b, 3 * NP * 8)) != nullptr;
     if (ok && b->n_general)
         ok = (b->general = (int2*)bdev_alloc(b, general.size() * sizeof(int2))) &&
              (b->gen_nodes = (int*)bdev_alloc(b, gen_nodes.size() * sizeof(int))) &&
@@ -2584,6 +2604,11 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
     } else {
         fill_insts<double>(b, P, instd);
         put(b->insts, instd.data(), instd.size() * sizeof(BatchInst<double>));
+        for (int i = 0; i < count && ce == cudaSuccess; ++i) {
+            bed_stencil_kernel<<<grid_blocks((size_t)b->nodes[i], 256, 4096), 256, 0, b->stream>>>(
+                instd[i].f[0], b->bed + b->off[i], NP);
+            ce = cudaGetLastError();
+        }
     }
     for (int k = 0; k < 2 && ce == cudaSuccess; ++k) {
         ce = cudaMemsetAsync(b->eta[k], 0, NP * b->esize, b->stream);

@@ -58,6 +58,14 @@ struct Coef {
     T Cb;    // C_b (Eq. bed-stress)
     T Om;    // Omega (Eq. SWE-force)
     T nz;    // -0.0, read at run time (see Op2::mul)
+    // FP64 form (derive64, update64): sums scaled by 3 e^2
+    T gh;    // g / 2
+    T i3e2;  // 1 / (3 e^2)
+    T i3e;   // 1 / (3 e)
+    T fwx;   // e dt / 2 times wfx, wfy, Cb, Om
+    T fwy;
+    T fCb;
+    T fOm;
 };
 
 template <typename T>
@@ -74,6 +82,8 @@ struct Fields {
     int idx32;    // 1 when pitch * ny < 2^31: node offsets fit in an int
     int edge[4];  // W, E, S, N
     Coef<T> c;
+    const T* bed;      // FP64: lambda-weighted stencils of D (sum, x- and y-moment; bed_stencil_kernel),
+    size_t bed_plane;  // three planes this many elements apart
 };
 
 template <typename T> struct Vec2;
@@ -94,6 +104,8 @@ struct Src {
     T o1, o2, o3, o4, o5, o6, o7, o8;
     T ownh;        // eta - h (5 G6 eta + 4 K6 |u|^2)
     T hFx, hFy;    // dt F / 2
+    // (FP64: o_a times 3 e^2, on the diagonals 12 e^2; ownh without eta and
+    // the force terms in the same units, see derive64)
 };
 
 template <typename T>
@@ -130,8 +142,31 @@ template <> struct Op<double> {
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-    static __device__ __forceinline__ double rcp(double a) { return 1.0 / a; }
-    static __device__ __forceinline__ double sqrt(double a) { return ::sqrt(a); }
+    // An FP64 warp instruction holds its SM quarter's pipe for 64 cycles, so
+    // these are written for few of them: the hardware's approximation (about
+    // 20 bits; it takes no FP64 slot) and one third-order step, which leaves
+    // an error of about an ulp.  With r = 1 - a y the reciprocal is
+    // y / (1 - r) = y (1 + r + r^2 + ...); with r = 1 - a y^2 the root is
+    // a y (1 - r)^(-1/2) = a y (1 + r / 2 + 3 r^2 / 8 + ...).
+    static __device__ __forceinline__ double rcp(double a)
+    {
+        const unsigned ex = (unsigned)__double2hiint(a) & 0x7fffffffu;
+        if (ex - 0x00200000u >= 0x7fa00000u) return 1.0 / a;  // zero, subnormal, huge, inf, nan (or their reciprocal)
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+        const double r = __fma_rn(-a, y, 1.0);
+        return __fma_rn(y, __fma_rn(r, r, r), y);
+    }
+    static __device__ __forceinline__ double sqrt(double a)
+    {
+        const unsigned ex = (unsigned)__double2hiint(a);
+        if (ex - 0x00100000u >= 0x7fe00000u)  // zero and subnormal: a root below 1.5e-154 is dropped; inf, nan
+            return ex < 0x00100000u ? 0.0 : (ex == 0x80000000u ? a : ::sqrt(a));
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+        const double q = __dmul_rn(a, y), r = __fma_rn(-q, y, 1.0);
+        return __fma_rn(__dmul_rn(q, r), __fma_rn(0.375, r, 0.5), q);
+    }
 };
 
 // Paired FP32 arithmetic on sm_100-class GPUs: one instruction applies the
@@ -179,10 +214,111 @@ __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
 // Which force terms of Eq. SWE-force are present (compile-time variants).
 enum : int { F_WIND = 1, F_FRICTION = 2, F_CORIOLIS = 4 };
 
+// Source-side quantities of one node in FP64.  The FP64 rate bounds every
+// FP64 step (fewer than two results per cycle and SM), so the sums are
+// arranged for few operations: all in units of 1 / (3 e^2), where
+//     3 e^2 a'  = g/2 h eta - (s + t) / 2,   s = h u^2, t = h v^2, w = h u v
+//     3 e^2 q'  = e h u + f,                 f = (e dt / 2) F
+// and with p = g/2 h eta + s - t/2 (= 3 e^2 (a' + s_xx)), d = p + 3 t / 2,
+// r = d - 3 s / 2 the outgoing values are p +- q_x, r +- q_y on the axes and
+// (d +- 3 w +- (q_x +- q_y)) / 4 on the diagonals, stored without the 1/4
+// (the receivers fold it into a multiply-add).  38 operations with friction
+// (root included), 46 and a longer root before; with update64 the tile
+// kernel's step of a 2999 x 701 channel went from 524 to 390 us, 0.93 of
+// what its operations take at the measured 19 cycles a warp instruction.
+template <int FM>
+__device__ __forceinline__ void derive64(const Coef<double>& c, const Raw<double>& r, Src<double>& s)
+{
+    using O = Op<double>;
+    double u = r.u, v = r.v, wx = c.fwx, wy = c.fwy, om = c.fOm;
+    if (r.flip) {  // specular ghost: normal components reversed, rotation sense too
+        if (r.flip & 1) { u = -u; wx = -wx; }
+        if (r.flip & 2) { v = -v; wy = -wy; }
+        if ((r.flip & 3) != 3) om = -om;
+    }
+    const double h = O::add(r.D, r.eta);
+    const double hu = O::mul(h, u), hv = O::mul(h, v);
+    const double sx = O::mul(hu, u), sy = O::mul(hv, v), sw = O::mul(hu, v);
+    const double ge = O::mul(O::mul(c.gh, r.eta), h);
+    const double p = O::add(O::fma(-0.5, sy, ge), sx);
+    const double d = O::fma(1.5, sy, p), q = O::fma(-1.5, sx, d);
+    s.ownh = O::fma(-2.0, d, O::mul(-3.0, ge));
+    double fx = (FM & F_WIND) ? wx : 0.0, fy = (FM & F_WIND) ? wy : 0.0;
+    if (FM & F_CORIOLIS) {
+        fx = O::fma(om, hv, fx);
+        fy = O::fma(-om, hu, fy);
+    }
+    if (FM & F_FRICTION) {
+        const double cs = O::mul(-c.fCb, O::sqrt(O::fma(u, u, O::mul(v, v))));
+        fx = O::fma(cs, u, fx);
+        fy = O::fma(cs, v, fy);
+    }
+    s.hFx = fx;
+    s.hFy = fy;
+    const double qx = FM ? O::fma(c.e, hu, fx) : O::mul(c.e, hu), qy = FM ? O::fma(c.e, hv, fy) : O::mul(c.e, hv);
+    s.o1 = O::add(p, qx);
+    s.o5 = O::sub(p, qx);
+    s.o3 = O::add(q, qy);
+    s.o7 = O::sub(q, qy);
+    const double dp = O::fma(3.0, sw, d), dm = O::fma(-3.0, sw, d);
+    const double s4 = O::add(qx, qy), t4 = O::sub(qx, qy);
+    s.o2 = O::add(dp, s4);
+    s.o6 = O::sub(dp, s4);
+    s.o8 = O::add(dm, t4);
+    s.o4 = O::sub(dm, t4);
+    s.eta = r.eta;
+    s.D = r.D;
+}
+
+// New eta, u, v of a node in FP64 from the eight incoming values (units of
+// derive64), the eta of its neighbours (m: row above, c: same row, p: row
+// below) and the stencils of D (bd: sum, x-moment, y-moment, precomputed,
+// since D is static): the streamed sums, then
+//     3 e^2 eta' = own + sum + g/2 (D S_eta - eta S_D),
+//     3 e hu'    = x-sum + g/2 (D X_eta - eta X_D) + 3 f_x.
+// 46 operations (56 and a division before).
+struct Bed64 {
+    double s, x, y;
+};
+struct Eta8 {
+    double mL, mC, mR, cL, cR, pL, pC, pR;
+};
+__device__ __forceinline__ void update64(const Coef<double>& K, double cL1, double mL2, double pL8, double cR5,
+                                         double mR4, double pR6, double mC3, double pC7, const Eta8& n, double eta,
+                                         double D, double own, double fx, double fy, const Bed64& bd, bool noslip,
+                                         double& oe, double& ou, double& ov)
+{
+    using O = Op<double>;
+    const double L = O::fma(0.25, O::add(mL2, pL8), cL1), R = O::fma(0.25, O::add(mR4, pR6), cR5);
+    const double Sh = O::add(O::add(L, R), O::add(mC3, pC7));
+    const double Sx = O::sub(L, R);
+    const double Sy = O::fma(0.25, O::sub(O::add(mL2, mR4), O::add(pL8, pR6)), O::sub(mC3, pC7));
+    const double EL = O::fma(0.25, O::add(n.mL, n.pL), n.cL), ER = O::fma(0.25, O::add(n.mR, n.pR), n.cR);
+    const double Es = O::add(O::add(EL, ER), O::add(n.mC, n.pC));
+    const double Ex = O::sub(EL, ER);
+    const double Ey = O::fma(0.25, O::sub(O::add(n.mL, n.mR), O::add(n.pL, n.pR)), O::sub(n.mC, n.pC));
+    const double Bs = O::fma(D, Es, O::mul(-eta, bd.s)), Bx = O::fma(D, Ex, O::mul(-eta, bd.x)),
+                 By = O::fma(D, Ey, O::mul(-eta, bd.y));
+    const double e1 = O::fma(K.i3e2, O::fma(K.gh, Bs, O::add(own, Sh)), eta);
+    const double mx = O::fma(3.0, fx, O::fma(K.gh, Bx, Sx)), my = O::fma(3.0, fy, O::fma(K.gh, By, Sy));
+    const double inv = O::mul(K.i3e, O::rcp(O::add(D, e1)));
+    oe = e1;
+    ou = noslip ? 0.0 : O::mul(mx, inv);
+    ov = noslip ? 0.0 : O::mul(my, inv);
+}
+__device__ __forceinline__ Bed64 bed_at(const Fields<double>& f, size_t i)
+{
+    return Bed64{f.bed[i], f.bed[i + f.bed_plane], f.bed[i + 2 * f.bed_plane]};
+}
+
 // Source-side quantities of one node (see the header comment).
 template <typename T, int FM>
 __device__ __forceinline__ void derive(const Coef<T>& c, const Raw<T>& r, Src<T>& s)
 {
+    if constexpr (std::is_same<T, double>::value) {
+        derive64<FM>(c, r, s);
+        return;
+    }
     using O = Op<T>;
     T u = r.u, v = r.v, wfx = c.wfx, wfy = c.wfy, Om = c.Om;
     if (r.flip) {  // specular ghost: normal components reversed, rotation sense too
@@ -330,6 +466,74 @@ __device__ __forceinline__ void derive2(const Coef2& c, const Raw<float>& r0, co
     s.o4 = P::sub(dm, t4);
     s.eta = eta;
     s.D = D;
+}
+
+// New eta, u, v of a node from its streamed sums (Sh, Sx, Sy: the first
+// terms of Eqs. Mac.lb.6 / Mac.lb.7 over the eight incoming outgoing values)
+// and the (eta, D) of its eight neighbours (m: row above, c: same row,
+// p: row below; L / C / R: column left / same / right), in the perturbation
+// form; eta, D, ownh, hFx, hFy are the node's own source quantities.  Every
+// kernel that updates fast-path nodes ends in this one function, so their
+// results agree bitwise.
+template <typename T, typename V2 = typename Vec2<T>::type>
+__device__ __forceinline__ void update_tail(const Coef<T>& K, T Sh, T Sx, T Sy, V2 mL, V2 mC, V2 mR, V2 cL, V2 cR,
+                                            V2 pL, V2 pC, V2 pR, T eta, T D, T ownh, T hFx, T hFy, bool noslip,
+                                            T& oe, T& ou, T& ov)
+{
+    using O = Op<T>;
+    const T q = T(0.25);
+    // lambda-weighted stencils of eta (.x) and D (.y): sum, x-moment, y-moment
+    T Se, Sd, Xe, Xd, Ye, Yd;
+#ifndef MACLAB_SCALAR_STENCIL
+    if constexpr (std::is_same<T, float>::value) {
+        // eta and D take the same operations: the two lanes of one paired
+        // instruction (each lane rounded as the scalar operation)
+        using P = Op2;
+        const float2 q2 = splat(q);
+        const float2 ML = P::fma(q2, P::add(mL, pL), cL), MR = P::fma(q2, P::add(mR, pR), cR);
+        const float2 S = P::add(P::add(ML, MR), P::add(mC, pC));
+        const float2 X = P::sub(ML, MR);
+        const float2 Y = P::fma(q2, P::sub(P::add(mL, mR), P::add(pL, pR)), P::sub(mC, pC));
+        Se = S.x, Sd = S.y, Xe = X.x, Xd = X.y, Ye = Y.x, Yd = Y.y;
+    } else
+#endif
+    {
+        const T MLe = O::fma(q, O::add(mL.x, pL.x), cL.x);
+        const T MRe = O::fma(q, O::add(mR.x, pR.x), cR.x);
+        const T MLd = O::fma(q, O::add(mL.y, pL.y), cL.y);
+        const T MRd = O::fma(q, O::add(mR.y, pR.y), cR.y);
+        Se = O::add(O::add(MLe, MRe), O::add(mC.x, pC.x));
+        Sd = O::add(O::add(MLd, MRd), O::add(mC.y, pC.y));
+        Xe = O::sub(MLe, MRe), Xd = O::sub(MLd, MRd);
+        Ye = O::fma(q, O::sub(O::add(mL.x, mR.x), O::add(pL.x, pR.x)), O::sub(mC.x, pC.x));
+        Yd = O::fma(q, O::sub(O::add(mL.y, mR.y), O::add(pL.y, pR.y)), O::sub(mC.y, pC.y));
+    }
+    const T A = O::mul(K.G6, D), B = O::mul(K.G6, eta);
+    // ownh already holds the receiver-only bed part 5 G6 eta_x D_x
+    const T eta1 = O::add(O::add(ownh, Sh), O::fma(A, Se, O::mul(-B, Sd)));
+    const T hu1 = O::fma(K.e, O::add(Sx, O::fma(A, Xe, O::mul(-B, Xd))), hFx);
+    const T hv1 = O::fma(K.e, O::add(Sy, O::fma(A, Ye, O::mul(-B, Yd))), hFy);
+    const T inv = O::rcp(O::add(D, eta1));
+    oe = eta1;
+    ou = noslip ? T(0) : O::mul(hu1, inv);
+    ov = noslip ? T(0) : O::mul(hv1, inv);
+}
+
+// Streamed sums of the first terms of Eqs. Mac.lb.6 / Mac.lb.7 from the
+// eight incoming values, grouped as (left column), (right column), centre:
+// a1 = cL_o1 + mL_o2 and a2 = cR_o5 + mR_o4 and sym = mL_o2 + mR_o4 + mC_o3
+// take only the node's own row and the row above, so a kernel that walks
+// down the rows can form them before the row below exists.
+template <typename T>
+__device__ __forceinline__ void streamed_sums(T a1, T a2, T sym, T mC_o3, T pL_o8, T pR_o6, T pC_o7, T& Sh, T& Sx,
+                                              T& Sy)
+{
+    using O = Op<T>;
+    const T OL = O::add(a1, pL_o8);
+    const T OR = O::add(a2, pR_o6);
+    Sh = O::add(O::add(OL, OR), O::add(mC_o3, pC_o7));
+    Sx = O::sub(OL, OR);
+    Sy = O::sub(sym, O::add(O::add(pL_o8, pR_o6), pC_o7));
 }
 
 // Map a column / row index outside the grid through the edge kinds.
@@ -557,34 +761,21 @@ __device__ __forceinline__ void emit_row(const Fields<T>& f, int j, int xl, int 
         const Src<T>& mL = m.col[k - 1]; const Src<T>& mC = m.col[k]; const Src<T>& mR = m.col[k + 1];
         const Src<T>& cL = c.col[k - 1]; const Src<T>& cC = c.col[k]; const Src<T>& cR = c.col[k + 1];
         const Src<T>& pL = p.col[k - 1]; const Src<T>& pC = p.col[k]; const Src<T>& pR = p.col[k + 1];
-        // streamed equilibria
-        const T OL = O::add(O::add(cL.o1, mL.o2), pL.o8);
-        const T OR = O::add(O::add(cR.o5, mR.o4), pR.o6);
-        const T Sh = O::add(O::add(OL, OR), O::add(mC.o3, pC.o7));
-        const T Sx = O::sub(OL, OR);
-        const T Sy = O::sub(O::add(O::add(mL.o2, mR.o4), mC.o3), O::add(O::add(pL.o8, pR.o6), pC.o7));
-        // lambda-weighted stencils of eta and D: sum, x-moment, y-moment
-        const T q = T(0.25);
-        const T MLe = O::fma(q, O::add(mL.eta, pL.eta), cL.eta);
-        const T MRe = O::fma(q, O::add(mR.eta, pR.eta), cR.eta);
-        const T MLd = O::fma(q, O::add(mL.D, pL.D), cL.D);
-        const T MRd = O::fma(q, O::add(mR.D, pR.D), cR.D);
-        const T Se = O::add(O::add(MLe, MRe), O::add(mC.eta, pC.eta));
-        const T Sd = O::add(O::add(MLd, MRd), O::add(mC.D, pC.D));
-        const T Xe = O::sub(MLe, MRe), Xd = O::sub(MLd, MRd);
-        const T Ye = O::fma(q, O::sub(O::add(mL.eta, mR.eta), O::add(pL.eta, pR.eta)), O::sub(mC.eta, pC.eta));
-        const T Yd = O::fma(q, O::sub(O::add(mL.D, mR.D), O::add(pL.D, pR.D)), O::sub(mC.D, pC.D));
-        const T etax = cC.eta, Dx = cC.D;
-        const T A = O::mul(K.G6, Dx), B = O::mul(K.G6, etax);
-        // ownh already holds the receiver-only bed part 5 G6 eta_x D_x
-        const T eta1 = O::add(O::add(cC.ownh, Sh), O::fma(A, Se, O::mul(-B, Sd)));
-        const T hu1 = O::fma(K.e, O::add(Sx, O::fma(A, Xe, O::mul(-B, Xd))), cC.hFx);
-        const T hv1 = O::fma(K.e, O::add(Sy, O::fma(A, Ye, O::mul(-B, Yd))), cC.hFy);
-        const T inv = O::rcp(O::add(Dx, eta1));
         const bool noslip = (ty & KIND_MASK) == K_NOSLIP;
-        oe[k - 1] = eta1;
-        ou[k - 1] = noslip ? T(0) : O::mul(hu1, inv);
-        ov[k - 1] = noslip ? T(0) : O::mul(hv1, inv);
+        if constexpr (std::is_same<T, double>::value) {
+            const size_t at = ok && j < f.ny ? (size_t)j * f.pitch + x : 0;
+            update64(K, cL.o1, mL.o2, pL.o8, cR.o5, mR.o4, pR.o6, mC.o3, pC.o7,
+                     Eta8{mL.eta, mC.eta, mR.eta, cL.eta, cR.eta, pL.eta, pC.eta, pR.eta}, cC.eta, cC.D, cC.ownh, cC.hFx,
+                     cC.hFy, bed_at(f, at), noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
+        } else {
+            using V2 = typename Vec2<T>::type;
+            auto ed = [](const Src<T>& q) { return V2{q.eta, q.D}; };
+            T Sh, Sx, Sy;
+            streamed_sums<T>(O::add(cL.o1, mL.o2), O::add(cR.o5, mR.o4), O::add(O::add(mL.o2, mR.o4), mC.o3), mC.o3,
+                             pL.o8, pR.o6, pC.o7, Sh, Sx, Sy);
+            update_tail<T>(K, Sh, Sx, Sy, ed(mL), ed(mC), ed(mR), ed(cL), ed(cR), ed(pL), ed(pC), ed(pR), cC.eta, cC.D,
+                           cC.ownh, cC.hFx, cC.hFy, noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
+        }
     }
     if (j >= f.ny || okmask == 0) return;
     const size_t row0 = (size_t)j * f.pitch;
@@ -769,9 +960,50 @@ __device__ __forceinline__ void general_finish(const Coef<T>& c, const NodeQ<T>&
 // the code is inlined into.  NEW: hbar at the new time level (Eq. h-bar as
 // written, hbar = (h(x, t + dt) + h(y, t)) / 2): the bed terms are linear in
 // the new eta of the node, which is then solved for directly.
+//
+// FP64 at the old level: a bounced link returns the node's own outgoing
+// value of the opposite direction, o_abar(x), without bed or force term.
+// That is the fast update with the source's (eta, D) replaced by the node's
+// own (the cross terms of the bed then cancel) and o_a(y) by o_abar(x),
+// whose source half of the force, lambda_a KF c_abar.F(x), cancels the
+// receiver half of that link.
+__device__ __forceinline__ void general_node64(const Fields<double>& f, int i, int j)
+{
+    const size_t xi = (size_t)j * f.pitch + i;
+    constexpr int ALL = F_WIND | F_FRICTION | F_CORIOLIS;
+    Src<double> X;
+    derive64<ALL>(f.c, Raw<double>{f.eta[xi], f.u[xi], f.v[xi], f.D[xi], 0}, X);
+    const double back[9] = {0.0, X.o5, X.o6, X.o7, X.o8, X.o1, X.o2, X.o3, X.o4};
+    double o[9], eta[9];
+#pragma unroll
+    for (int a = 1; a < 9; ++a) {
+        const int cx = (a == 1 || a == 2 || a == 8) - (a == 4 || a == 5 || a == 6);
+        const int cy = (a >= 2 && a <= 4) - (a >= 6);
+        uint8_t flip = 0;
+        const int si = resolve_index(i - cx, f.nx, f.edge[0], f.edge[1], 1, flip);
+        const int sj = resolve_index(j - cy, f.ny, f.edge[2], f.edge[3], 2, flip);
+        o[a] = back[a];
+        eta[a] = X.eta;
+        if (si < 0 || sj < 0) continue;
+        const size_t s = (size_t)sj * f.pitch + si;
+        if ((f.type[s] & KIND_MASK) == K_SOLID) continue;
+        Src<double> Y;
+        derive64<ALL>(f.c, Raw<double>{f.eta[s], f.u[s], f.v[s], f.D[s], flip}, Y);
+        o[a] = a == 1 ? Y.o1 : a == 2 ? Y.o2 : a == 3 ? Y.o3 : a == 4 ? Y.o4 : a == 5 ? Y.o5 : a == 6 ? Y.o6 : a == 7 ? Y.o7 : Y.o8;
+        eta[a] = Y.eta;
+    }
+    update64(f.c, o[1], o[2], o[8], o[5], o[4], o[6], o[3], o[7],
+             Eta8{eta[2], eta[3], eta[4], eta[1], eta[5], eta[8], eta[7], eta[6]}, X.eta, X.D, X.ownh, X.hFx, X.hFy,
+             bed_at(f, xi), (f.type[xi] & KIND_MASK) == K_NOSLIP, f.eta1[xi], f.u1[xi], f.v1[xi]);
+}
+
 template <typename T, bool NEW = false>
 __device__ __forceinline__ void general_node(const Fields<T>& f, int i, int j)
 {
+    if constexpr (std::is_same<T, double>::value && !NEW) {
+        general_node64(f, i, j);
+        return;
+    }
     using O = Op<T>;
     const size_t xi = (size_t)j * f.pitch + i;
     const Coef<T>& c = f.c;
@@ -835,6 +1067,34 @@ __global__ void __launch_bounds__(128) step_general_kernel(const Fields<T> f, co
     if (t >= count) return;
     const int node = list[t];
     general_node<T, NEW>(f, node % f.nx, node / f.nx);
+}
+
+// Stencils of the still-water depth for the FP64 update (once per grid): sum,
+// x- and y-moment of lambda_a D(x - c_a), a bounced link's source depth being
+// the node's own.
+static __global__ void bed_stencil_kernel(const __grid_constant__ Fields<double> f, double* __restrict__ bed,
+                                          size_t plane)
+{
+    using O = Op<double>;
+    const size_t total = (size_t)f.nx * f.ny;
+    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < total; k += (size_t)gridDim.x * blockDim.x) {
+        const int j = (int)(k / f.nx), i = (int)(k - (size_t)j * f.nx);
+        const size_t x = (size_t)j * f.pitch + i;
+        double d[9];
+        for (int a = 1; a < 9; ++a) {
+            uint8_t flip = 0;
+            const int si = resolve_index(i - c_cx[a], f.nx, f.edge[0], f.edge[1], 1, flip);
+            const int sj = resolve_index(j - c_cy[a], f.ny, f.edge[2], f.edge[3], 2, flip);
+            d[a] = f.D[x];
+            if (si < 0 || sj < 0) continue;
+            const size_t s = (size_t)sj * f.pitch + si;
+            if ((f.type[s] & KIND_MASK) != K_SOLID) d[a] = f.D[s];
+        }
+        const double L = O::fma(0.25, O::add(d[2], d[8]), d[1]), R = O::fma(0.25, O::add(d[4], d[6]), d[5]);
+        bed[x] = O::add(O::add(L, R), O::add(d[3], d[7]));
+        bed[x + plane] = O::sub(L, R);
+        bed[x + 2 * plane] = O::fma(0.25, O::sub(O::add(d[2], d[4]), O::add(d[8], d[6])), O::sub(d[3], d[7]));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1104,82 +1364,22 @@ __device__ __forceinline__ void tile_phase_a(const Fields<T>& f, int x0, int y0,
     }
 }
 
-// New eta, u, v of a node from its streamed sums (Sh, Sx, Sy: the first
-// terms of Eqs. Mac.lb.6 / Mac.lb.7 over the eight incoming outgoing values)
-// and the (eta, D) of its eight neighbours (m: row above, c: same row,
-// p: row below; L / C / R: column left / same / right), in the perturbation
-// form; eta, D, ownh, hFx, hFy are the node's own source quantities.  Every
-// kernel that updates fast-path nodes ends in this one function, so their
-// results agree bitwise.
-template <typename T, typename V2 = typename Vec2<T>::type>
-__device__ __forceinline__ void update_tail(const Coef<T>& K, T Sh, T Sx, T Sy, V2 mL, V2 mC, V2 mR, V2 cL, V2 cR,
-                                            V2 pL, V2 pC, V2 pR, T eta, T D, T ownh, T hFx, T hFy, bool noslip,
-                                            T& oe, T& ou, T& ov)
-{
-    using O = Op<T>;
-    const T q = T(0.25);
-    // lambda-weighted stencils of eta (.x) and D (.y): sum, x-moment, y-moment
-    T Se, Sd, Xe, Xd, Ye, Yd;
-#ifndef MACLAB_SCALAR_STENCIL
-    if constexpr (std::is_same<T, float>::value) {
-        // eta and D take the same operations: the two lanes of one paired
-        // instruction (each lane rounded as the scalar operation)
-        using P = Op2;
-        const float2 q2 = splat(q);
-        const float2 ML = P::fma(q2, P::add(mL, pL), cL), MR = P::fma(q2, P::add(mR, pR), cR);
-        const float2 S = P::add(P::add(ML, MR), P::add(mC, pC));
-        const float2 X = P::sub(ML, MR);
-        const float2 Y = P::fma(q2, P::sub(P::add(mL, mR), P::add(pL, pR)), P::sub(mC, pC));
-        Se = S.x, Sd = S.y, Xe = X.x, Xd = X.y, Ye = Y.x, Yd = Y.y;
-    } else
-#endif
-    {
-        const T MLe = O::fma(q, O::add(mL.x, pL.x), cL.x);
-        const T MRe = O::fma(q, O::add(mR.x, pR.x), cR.x);
-        const T MLd = O::fma(q, O::add(mL.y, pL.y), cL.y);
-        const T MRd = O::fma(q, O::add(mR.y, pR.y), cR.y);
-        Se = O::add(O::add(MLe, MRe), O::add(mC.x, pC.x));
-        Sd = O::add(O::add(MLd, MRd), O::add(mC.y, pC.y));
-        Xe = O::sub(MLe, MRe), Xd = O::sub(MLd, MRd);
-        Ye = O::fma(q, O::sub(O::add(mL.x, mR.x), O::add(pL.x, pR.x)), O::sub(mC.x, pC.x));
-        Yd = O::fma(q, O::sub(O::add(mL.y, mR.y), O::add(pL.y, pR.y)), O::sub(mC.y, pC.y));
-    }
-    const T A = O::mul(K.G6, D), B = O::mul(K.G6, eta);
-    // ownh already holds the receiver-only bed part 5 G6 eta_x D_x
-    const T eta1 = O::add(O::add(ownh, Sh), O::fma(A, Se, O::mul(-B, Sd)));
-    const T hu1 = O::fma(K.e, O::add(Sx, O::fma(A, Xe, O::mul(-B, Xd))), hFx);
-    const T hv1 = O::fma(K.e, O::add(Sy, O::fma(A, Ye, O::mul(-B, Yd))), hFy);
-    const T inv = O::rcp(O::add(D, eta1));
-    oe = eta1;
-    ou = noslip ? T(0) : O::mul(hu1, inv);
-    ov = noslip ? T(0) : O::mul(hv1, inv);
-}
-
-// Streamed sums of the first terms of Eqs. Mac.lb.6 / Mac.lb.7 from the
-// eight incoming values, grouped as (left column), (right column), centre:
-// a1 = cL_o1 + mL_o2 and a2 = cR_o5 + mR_o4 and sym = mL_o2 + mR_o4 + mC_o3
-// take only the node's own row and the row above, so a kernel that walks
-// down the rows can form them before the row below exists.
-template <typename T>
-__device__ __forceinline__ void streamed_sums(T a1, T a2, T sym, T mC_o3, T pL_o8, T pR_o6, T pC_o7, T& Sh, T& Sx,
-                                              T& Sy)
-{
-    using O = Op<T>;
-    const T OL = O::add(a1, pL_o8);
-    const T OR = O::add(a2, pR_o6);
-    Sh = O::add(O::add(OL, OR), O::add(mC_o3, pC_o7));
-    Sx = O::sub(OL, OR);
-    Sy = O::sub(sym, O::add(O::add(pL_o8, pR_o6), pC_o7));
-}
-
 // New eta, u, v of the node at tile row lr, column lc from the derived values
 // of its eight neighbours in shared memory (Eqs. Mac.lb.6 / Mac.lb.7 in the
 // perturbation form); eta, D, ownh, hFx, hFy are the node's own source
 // quantities.
 template <typename T, typename DR>
 __device__ __forceinline__ void node_update(const DR& sm, int lr, int lc, const Coef<T>& K, T eta, T D, T ownh,
-                                            T hFx, T hFy, bool noslip, T& oe, T& ou, T& ov)
+                                            T hFx, T hFy, bool noslip, const Bed64& bd, T& oe, T& ou, T& ov)
 {
+    if constexpr (std::is_same<T, double>::value) {
+        update64(K, sm.o(0, lr, lc - 1), sm.o(1, lr - 1, lc - 1), sm.o(7, lr + 1, lc - 1), sm.o(4, lr, lc + 1),
+                 sm.o(3, lr - 1, lc + 1), sm.o(5, lr + 1, lc + 1), sm.o(2, lr - 1, lc), sm.o(6, lr + 1, lc),
+                 Eta8{sm.ed(lr - 1, lc - 1).x, sm.ed(lr - 1, lc).x, sm.ed(lr - 1, lc + 1).x, sm.ed(lr, lc - 1).x,
+                      sm.ed(lr, lc + 1).x, sm.ed(lr + 1, lc - 1).x, sm.ed(lr + 1, lc).x, sm.ed(lr + 1, lc + 1).x},
+                 eta, D, ownh, hFx, hFy, bd, noslip, oe, ou, ov);
+        return;
+    }
     using O = Op<T>;
     const T cL_o1 = sm.o(0, lr, lc - 1), mL_o2 = sm.o(1, lr - 1, lc - 1), pL_o8 = sm.o(7, lr + 1, lc - 1);
     const T cR_o5 = sm.o(4, lr, lc + 1), mR_o4 = sm.o(3, lr - 1, lc + 1), pR_o6 = sm.o(5, lr + 1, lc + 1);
@@ -1219,8 +1419,10 @@ __device__ __forceinline__ void tile_phase_bc(const Fields<T>& f, int x0, int y0
             const bool ok = (inside || (x < f.nx && y < f.ny)) && (ty & KIND_MASK) != K_SOLID && !(ty & GENERAL_BIT);
             okmask |= (ok ? 1u : 0u) << k;
             const Src<T>& me = own[r][k];
+            Bed64 bd{};
+            if constexpr (std::is_same<T, double>::value) bd = bed_at(f, ok ? (size_t)y * f.pitch + x : 0);
             node_update<T>(sm, lr, lc, K, me.eta, me.D, me.ownh, me.hFx, me.hFy,
-                           (ty & KIND_MASK) == K_NOSLIP, oe[k], ou[k], ov[k]);
+                           (ty & KIND_MASK) == K_NOSLIP, bd, oe[k], ou[k], ov[k]);
         }
         if (okmask == 0) continue;
         const size_t idx = inside ? (size_t)(y * f.pitch + x0 + 2 * tx) : (size_t)y * f.pitch + x0 + 2 * tx;
@@ -1435,7 +1637,7 @@ __device__ __forceinline__ void window_node(const tile2::Smem& sm, const Coef<fl
     const float2 oh = sm.own[0][r][j], fx = sm.own[1][r][j], fy = sm.own[2][r][j];
     const uint8_t ty = (uint8_t)(sm.type[r][j] >> (8 * k));
     node_update<float>(sm.d, r, c, K, ed.x, ed.y, k ? oh.y : oh.x, k ? fx.y : fx.x, k ? fy.y : fy.x,
-                       (ty & KIND_MASK) == K_NOSLIP, oe, ou, ov);
+                       (ty & KIND_MASK) == K_NOSLIP, Bed64{}, oe, ou, ov);
 }
 
 // f: eta, u, v at step n; eta1, u1, v1 the step-n+1 buffer (outer ring only);

@@ -408,16 +408,13 @@ __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, cons
             gather_pair(c2, A1, M2, C5, M4, M3, V2{Lo8, d.o8.x}, V2{d.o6.y, Ro6}, d.o7, m, c, pe, own.ownh,
                         own.hFx, own.hFy, ns0, ns1, oe, ou, ov);
         } else {
-            using O = Op<T>;
-            T Sh, Sx, Sy;
-            streamed_sums<T>(O::add(A1.x, M2.x), O::add(C5.x, M4.x), O::add(O::add(M2.x, M4.x), M3.x), M3.x, Lo8,
-                             d.o6.y, d.o7.x, Sh, Sx, Sy);
-            update_tail<T>(f.c, Sh, Sx, Sy, m[0], m[1], m[2], c[0], c[2], pe[0], pe[1], pe[2], c[1].x, c[1].y,
-                           own.ownh.x, own.hFx.x, own.hFy.x, ns0, oe.x, ou.x, ov.x);
-            streamed_sums<T>(O::add(A1.y, M2.y), O::add(C5.y, M4.y), O::add(O::add(M2.y, M4.y), M3.y), M3.y,
-                             d.o8.x, Ro6, d.o7.y, Sh, Sx, Sy);
-            update_tail<T>(f.c, Sh, Sx, Sy, m[1], m[2], m[3], c[1], c[3], pe[1], pe[2], pe[3], c[2].x, c[2].y,
-                           own.ownh.y, own.hFx.y, own.hFy.y, ns1, oe.y, ou.y, ov.y);
+            const size_t at = EDGE ? (size_t)(r - 1) * f.pitch + x : (size_t)(unsigned)((r - 1) * f.pitch + x);
+            update64(f.c, A1.x, M2.x, Lo8, C5.x, M4.x, d.o6.y, M3.x, d.o7.x,
+                     Eta8{m[0].x, m[1].x, m[2].x, c[0].x, c[2].x, pe[0].x, pe[1].x, pe[2].x}, c[1].x, c[1].y, own.ownh.x,
+                     own.hFx.x, own.hFy.x, bed_at(f, ok & 1u ? at : 0), ns0, oe.x, ou.x, ov.x);
+            update64(f.c, A1.y, M2.y, d.o8.x, C5.y, M4.y, Ro6, M3.y, d.o7.y,
+                     Eta8{m[1].x, m[2].x, m[3].x, c[1].x, c[3].x, pe[1].x, pe[2].x, pe[3].x}, c[2].x, c[2].y, own.ownh.y,
+                     own.hFx.y, own.hFy.y, bed_at(f, ok & 2u ? at + 1 : 0), ns1, oe.y, ou.y, ov.y);
         }
         const size_t idx = EDGE ? (size_t)(r - 1) * f.pitch + x : (size_t)(unsigned)((r - 1) * f.pitch + x);
         if (!EDGE && OUT == 60) {

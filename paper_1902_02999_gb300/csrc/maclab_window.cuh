@@ -21,17 +21,18 @@
 // One step, old raw state in buffer s & 1:
 //   A  every node of the region derives its source quantities (derive2 /
 //      derive) into shared memory; ghosts likewise, with their flips;
-//   B  every fast node gathers and updates (gather_pair / update_tail) into
-//      the other raw buffer; a node with a bounce-back link is updated by
-//      eight lanes, one link each, its sums added in the order of
-//      general_node;
+//   B  every fast node gathers and updates (gather_pair / update64) into
+//      the other raw buffer; a node with a bounce-back link reads its own
+//      outgoing values for the bounced links (FP64, as general_node64) or is
+//      updated by eight lanes, one link each, its sums added in the order of
+//      general_node (FP32);
 //   C  Dirichlet nodes take their values from the new inward node.
 // Every node takes the operations of the single-step kernels in their
 // order, so the states are bitwise theirs.
 //
 // Measured per step, single-step launches (graph replay where the boundary
 // is steady) -> this kernel: 256 x 256 lake FP32 11.4 -> 3.3 us, 400 x 3
-// tidal strip FP64 49 -> 10 us, eight 256 x 256 lakes FP64 195 -> 113 us.
+// tidal strip FP64 49 -> 5.4 us, eight 256 x 256 lakes FP64 195 -> 70 us.
 #pragma once
 #include "maclab_march.cuh"
 
@@ -99,8 +100,9 @@ struct Arrays<double> {
     double* own;     // [3][rows][2 hw]: ownh, hFx, hFy
     double* raws;
     double* D;
+    double* bed;     // [3][rows][2 hw]: stencils of D
     Dir* dir;
-    uint8_t* type;
+    uint16_t* type;  // type byte | bounced links << 8 (bit a - 1: direction a)
     uint16_t* list;
     int hw, rows;
     __device__ __forceinline__ int plane() const { return rows * 2 * hw; }
@@ -108,11 +110,11 @@ struct Arrays<double> {
 };
 
 template <typename T>
-__host__ __device__ constexpr size_t cell_bytes() { return sizeof(T) == 4 ? 68 : 144; }
+__host__ __device__ constexpr size_t cell_bytes() { return sizeof(T) == 4 ? 68 : 168; }
 __host__ __device__ inline size_t smem_of(size_t per_cell, const Shape& s)
 {
     const size_t cells = (size_t)s.rows * 2 * s.hw;
-    return cells * per_cell + (size_t)s.ndir * sizeof(Dir) + ((cells + 15) & ~size_t(15)) +
+    return cells * per_cell + (size_t)s.ndir * sizeof(Dir) + ((cells + 15) & ~size_t(15)) * (per_cell > 100 ? 2 : 1) +
            (((size_t)s.nlist * 2 + 15) & ~size_t(15));
 }
 
@@ -135,8 +137,13 @@ __device__ __forceinline__ Arrays<T> carve(unsigned char* p, const Shape& s)
         a.raws = a.own + 3 * n;
     }
     a.D = a.raws + 6 * n;
-    a.dir = reinterpret_cast<Dir*>(a.D + n);
-    a.type = reinterpret_cast<uint8_t*>(a.dir + s.ndir);
+    T* end = a.D + n;
+    if constexpr (std::is_same<T, double>::value) {
+        a.bed = end;
+        end += 3 * n;
+    }
+    a.dir = reinterpret_cast<Dir*>(end);
+    a.type = reinterpret_cast<decltype(a.type)>(a.dir + s.ndir);
     a.list = reinterpret_cast<uint16_t*>(a.type + ((n + 15) & ~15));
     return a;
 }
@@ -351,6 +358,12 @@ step_window_kernel(const BatchInst<T>* __restrict__ insts, const window::Item* _
         A.D[cell] = f.D[g];
         A.type[cell] = ty;
         const int kind = ty & KIND_MASK;
+        if constexpr (std::is_same<T, double>::value) {
+            const Bed64 b = bed_at(f, g);
+            A.bed[cell] = b.s;
+            A.bed[n + cell] = b.x;
+            A.bed[2 * n + cell] = b.y;
+        }
         if (ty & GENERAL_BIT) {
             A.list[atomicAdd(&counts[0], 1)] = (uint16_t)cell;
         } else if (kind >= K_DIR_H) {
@@ -362,13 +375,21 @@ step_window_kernel(const BatchInst<T>* __restrict__ insts, const window::Item* _
     }
     const int nghost = 2 * (ax.n + 2) + 2 * ay.n;
     if constexpr (std::is_same<T, double>::value) {
-        // ghosts keep their still-water depth; eta follows every step
+        // bounced links of the listed nodes
         __syncthreads();
-        for (int q = tid; q < nghost; q += nt) {
-            int col, row, sc, sr;
-            uint8_t flip;
-            if (ghost(ax, ay, q, col, row, sc, sr, flip))
-                A.D[(row + 1) * pw + col + 2] = A.D[(sr + 1) * pw + sc + 2];
+        for (int g = tid; g < counts[0]; g += nt) {
+            const int cell = A.list[g], pr = cell / pw, pc = cell - pr * pw;
+            uint32_t mask = 0;
+#pragma unroll
+            for (int a = 1; a < 9; ++a) {
+                const int cx = (a == 1 || a == 2 || a == 8) - (a == 4 || a == 5 || a == 6);
+                const int cy = (a >= 2 && a <= 4) - (a >= 6);
+                uint8_t flip = 0;
+                const int sc = resolve(ax, pc - 2 - cx, flip), sr = resolve(ay, pr - 1 - cy, flip);
+                const bool back = sc < 0 || sr < 0 || (A.type[(sr + 1) * pw + sc + 2] & KIND_MASK) == K_SOLID;
+                mask |= (back ? 1u : 0u) << (a - 1);
+            }
+            A.type[cell] |= (uint16_t)(mask << 8);
         }
     }
     // FP32: the thread's pairs, fixed for the launch
@@ -475,26 +496,29 @@ step_window_kernel(const BatchInst<T>* __restrict__ insts, const window::Item* _
             for (int p = tid; p < cells; p += nt) {
                 const int r = e0 + p / w, q = (r + 1) * pw + d0 + p % w + 2;
                 const uint32_t ty = A.type[q];
-                if (ty - 1u >= 7u) continue;  // solid, or a bounce-back link
-                using V2 = typename Vec2<T>::type;
-                const T* o = A.o;
-                const T cL1 = o[q - 1], mL2 = o[n + q - pw - 1], pL8 = o[7 * n + q + pw - 1];
-                const T cR5 = o[4 * n + q + 1], mR4 = o[3 * n + q - pw + 1], pR6 = o[5 * n + q + pw + 1];
-                const T mC3 = o[2 * n + q - pw], pC7 = o[6 * n + q + pw];
-                using O = Op<T>;
-                T Sh, Sx, Sy, oe, ou, ov;
-                streamed_sums<T>(O::add(cL1, mL2), O::add(cR5, mR4), O::add(O::add(mL2, mR4), mC3), mC3, pL8, pR6, pC7,
-                                 Sh, Sx, Sy);
-                auto ed = [&](int i) { return V2{raw[i], A.D[i]}; };
-                update_tail<T>(c, Sh, Sx, Sy, ed(q - pw - 1), ed(q - pw), ed(q - pw + 1), ed(q - 1), ed(q + 1),
-                               ed(q + pw - 1), ed(q + pw), ed(q + pw + 1), raw[q], A.D[q], A.own[q], A.own[n + q],
-                               A.own[2 * n + q], (ty & KIND_MASK) == K_NOSLIP, oe, ou, ov);
+                if ((ty & KIND_MASK) == K_SOLID) continue;
+                // where each link reads: the neighbour, or for a bounced link
+                // the node itself, opposite direction
+                const int nb[8] = {q - 1, q - pw - 1, q - pw, q - pw + 1, q + 1, q + pw + 1, q + pw, q + pw - 1};
+                const uint32_t mask = ty >> 8;
+                double o[8], eta[8];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    const bool back = (mask >> a) & 1u;
+                    o[a] = A.o[back ? ((a + 4) & 7) * n + q : a * n + nb[a]];
+                    eta[a] = raw[back ? q : nb[a]];
+                }
+                T oe, ou, ov;
+                update64(c, o[0], o[1], o[7], o[4], o[3], o[5], o[2], o[6],
+                         Eta8{eta[1], eta[2], eta[3], eta[0], eta[4], eta[7], eta[6], eta[5]}, raw[q], A.D[q], A.own[q],
+                         A.own[n + q], A.own[2 * n + q], Bed64{A.bed[q], A.bed[n + q], A.bed[2 * n + q]},
+                         (ty & KIND_MASK) == K_NOSLIP, oe, ou, ov);
                 nxt[q] = oe;
                 nxt[n + q] = ou;
                 nxt[2 * n + q] = ov;
             }
         }
-        for (int g = tid >> 3; g < ng; g += nt >> 3) {
+        for (int g = tid >> 3; g < (std::is_same<T, double>::value ? 0 : ng); g += nt >> 3) {
             const int cell = A.list[g], r = cell / pw - 1, q = cell - (r + 1) * pw - 2;
             if (r < e0 || r >= e1 || q < d0 || q >= d1) continue;  // the group's eight lanes alike
             T oe, ou, ov;

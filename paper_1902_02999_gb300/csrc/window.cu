@@ -20,7 +20,7 @@ constexpr double LAUNCH_CYCLES = 5000;      // launch, dependent loads, store
 constexpr double LOAD_CELL = 1.0;           // per window node loaded
 constexpr double STEP_CYCLES = 500;         // barriers and the latency of one step
 constexpr double CELL_F32 = 1.1;            // per node and step
-constexpr double INSTR_F64 = 118;           // FP64 instructions per node and step
+constexpr double INSTR_F64 = 86;            // FP64 instructions per node and step
 
 // nodes that are not solid in [0, x) x [0, y), row length nx + 1
 struct Counts {
