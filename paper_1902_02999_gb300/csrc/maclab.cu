@@ -116,7 +116,7 @@ struct maclab_s {
     // several steps per launch (small grids; maclab_window.cuh)
     bool kernel_chosen = false;    // the caller picked a step kernel: every step is a launch of it
     window::Plan wplan;            // k = 0: not used on this grid
-    window::Item* witems = nullptr;
+    window::Lists wlists{};
     void* winst = nullptr;         // BatchInst<T>[1]
     void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches
     std::vector<cudaEvent_t> events;  // pairs around step-kernel launches
@@ -515,11 +515,15 @@ struct WindowRun {
 // before the last step in other.
 template <typename T>
 window::Buffers<T> window_buffers(const WindowRun& r, int64_t i, void* const (&eta)[2], void* const (&u)[2],
-                                  void* const (&v)[2], void* const (&mid)[3], int cur)
+                                  void* const (&v)[2], void* const (&mid)[3], int cur, const void* D, const void* bed,
+                                  size_t plane)
 {
     void* A[3] = {eta[cur], u[cur], v[cur]};
     void* B[3] = {eta[1 - cur], u[1 - cur], v[1 - cur]};
     window::Buffers<T> b{};
+    b.D = (const T*)D;
+    b.bed = (const T*)bed;
+    b.plane = plane;
     for (int q = 0; q < 3; ++q) {
         b.in[q] = (const T*)(i == 0 ? A[q] : r.to_scratch(i - 1) ? mid[q] : B[q]);
         if (r.launches == 1) {
@@ -538,6 +542,7 @@ template <typename T>
 int advance_window(maclab_t s, int64_t n)
 {
     const WindowRun r(n, s->wplan.k);
+    int64_t done = 0;
     for (int64_t i = 0; i < r.launches; ++i) {
         const int steps = r.steps(i);
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -556,14 +561,16 @@ int advance_window(maclab_t s, int64_t n)
         window::DirTable tab;
         const bool steady = s->steady_bc || s->n_dir == 0;
         if (!steady)
-            for (int k = 0; k < steps; ++k) tab.v[k] = dir_values(s, s->n + k + 1);
-        const cudaError_t e = window::launch<T>(s->wplan, s->winst, s->witems, nullptr,
-                                                window_buffers<T>(r, i, s->eta, s->u, s->v, s->wmid, s->cur), steps,
-                                                steady ? nullptr : &tab, s->stream);
+            for (int k = 0; k < steps; ++k) tab.v[k] = dir_values(s, s->n + done + k + 1);
+        const cudaError_t e = window::launch<T>(
+            s->wplan, s->winst, s->wlists, nullptr,
+            window_buffers<T>(r, i, s->eta, s->u, s->v, s->wmid, s->cur, s->D, s->bed, (size_t)s->pitch * s->grid.ny), steps,
+            steady ? nullptr : &tab, s->stream);
         if (e != cudaSuccess) return cuda_fail(s, e, "step launch");
         if (s->profiling) cudaEventRecord(ev1, s->stream);
-        s->n += steps;
+        done += steps;
     }
+    s->n += n;
     if (r.launches == 1) s->cur = 1 - s->cur;
     s->have_prev = true;
     return MACLAB_OK;
@@ -1106,12 +1113,12 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     const bool f64 = s->prec == MACLAB_F64;
     s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0}}, f64, s->fmode, sms);
     if (s->wplan.k == 0) return MACLAB_OK;
-    const size_t NP = (size_t)P.pitch * P.ny, items = s->wplan.items.size() * sizeof(window::Item);
-    bool ok = (s->witems = (window::Item*)dev_alloc(s, items)) != nullptr &&
-              (s->winst = dev_alloc(s, f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>))) != nullptr;
+    const size_t NP = (size_t)P.pitch * P.ny;
+    void* mem = dev_alloc(s, window::list_bytes(s->wplan));
+    bool ok = mem != nullptr && (s->winst = dev_alloc(s, f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>))) != nullptr;
     for (int q = 0; q < 3 && ok; ++q) ok = (s->wmid[q] = dev_alloc(s, NP * s->esize)) != nullptr;
     if (!ok) return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
-    cudaError_t e = cudaMemcpyAsync(s->witems, s->wplan.items.data(), items, cudaMemcpyHostToDevice, s->stream);
+    cudaError_t e = cudaSuccess;
     BatchInst<float> f{};
     BatchInst<double> d{};
     if (f64) d = make_inst<double>(P, s->eta, s->u, s->v, s->D, s->D64, s->type, s->bed, NP, 0);
@@ -1119,7 +1126,9 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     if (e == cudaSuccess)
         e = f64 ? cudaMemcpyAsync(s->winst, &d, sizeof(d), cudaMemcpyHostToDevice, s->stream)
                 : cudaMemcpyAsync(s->winst, &f, sizeof(f), cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) e = window::prepare_launch(s->wplan, f64);
+    if (e == cudaSuccess)
+        e = f64 ? window::build_lists<double>(s->wplan, s->winst, mem, s->stream, &s->wlists)
+                : window::build_lists<float>(s->wplan, s->winst, mem, s->stream, &s->wlists);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "upload");
     return MACLAB_OK;
@@ -2196,7 +2205,7 @@ struct maclab_batch_s {
     bool broken = false;            // a persistent step stopped early: the state must be reloaded
     std::vector<uint8_t> reloaded;  // instances set since the batch broke
     window::Plan wplan;             // several steps per launch (k = 0: not used)
-    window::Item* witems = nullptr;
+    window::Lists wlists{};
     void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches, packed
     void* snap[3] = {nullptr, nullptr, nullptr};  // marked state, packed like eta / u / v
     int64_t mark_n = -1;            // step count of the marked state (-1: none)
@@ -2358,8 +2367,9 @@ int batch_window(maclab_batch_t b, int64_t n, cudaStream_t st)
     const WindowRun r(n, b->wplan.k);
     for (int64_t i = 0; i < r.launches; ++i) {
         const cudaError_t e =
-            window::launch<T>(b->wplan, b->insts, b->witems, b->active,
-                              window_buffers<T>(r, i, b->eta, b->u, b->v, b->wmid, b->cur), r.steps(i), nullptr, st);
+            window::launch<T>(b->wplan, b->insts, b->wlists, b->active,
+                              window_buffers<T>(r, i, b->eta, b->u, b->v, b->wmid, b->cur, b->D, b->bed, b->total_np),
+                              r.steps(i), nullptr, st);
         if (e != cudaSuccess) return bfail(b, MACLAB_E_CUDA, std::string("batch step launch: ") + cudaGetErrorString(e));
     }
     if (r.launches == 1) b->cur = 1 - b->cur;
@@ -2641,16 +2651,16 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         b->wplan = window::make_plan(views, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
         if (b->wplan.k > 0) {
-            const size_t bytes = b->wplan.items.size() * sizeof(window::Item);
-            bool got = (b->witems = (window::Item*)bdev_alloc(b, bytes)) != nullptr;
+            void* mem = bdev_alloc(b, window::list_bytes(b->wplan));
+            bool got = mem != nullptr;
             for (int q = 0; q < 3 && got; ++q) got = (b->wmid[q] = bdev_alloc(b, NP * b->esize)) != nullptr;
             if (!got) {
                 brelease(b);
                 delete b;
                 return bfail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
             }
-            ce = cudaMemcpyAsync(b->witems, b->wplan.items.data(), bytes, cudaMemcpyHostToDevice, b->stream);
-            if (ce == cudaSuccess) ce = window::prepare_launch(b->wplan, b->prec == MACLAB_F64);
+            ce = b->prec == MACLAB_F32 ? window::build_lists<float>(b->wplan, b->insts, mem, b->stream, &b->wlists)
+                                       : window::build_lists<double>(b->wplan, b->insts, mem, b->stream, &b->wlists);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
             if (ce != cudaSuccess) {
                 bfail(nullptr, MACLAB_E_CUDA, std::string("batch upload: ") + cudaGetErrorString(ce));

@@ -3,7 +3,7 @@
 #include "window.h"
 
 #include <algorithm>
-#include <cstring>
+#include <cmath>
 
 namespace maclab {
 namespace window {
@@ -15,12 +15,28 @@ namespace {
 
 constexpr size_t MAX_SMEM = 227 * 1024 - 2048;
 
-// Cost model in SM cycles.
-constexpr double LAUNCH_CYCLES = 5000;      // launch, dependent loads, store
-constexpr double LOAD_CELL = 1.0;           // per window node loaded
-constexpr double STEP_CYCLES = 500;         // barriers and the latency of one step
-constexpr double CELL_F32 = 1.1;            // per node and step
-constexpr double INSTR_F64 = 86;            // FP64 instructions per node and step
+// Cost model in SM cycles, fitted to clock readings inside the kernel and to
+// whole runs on a GB300 (2.07 GHz): 256 x 256 lake, 1001 x 333 channel,
+// 400 x 3 strip.
+constexpr double LAUNCH_CYCLES = 4000;  // launch
+constexpr double BLOCK_CYCLES = 4500;   // a block's dependent loads and its store
+constexpr double LOAD_CELL = 1.5;       // per window node
+constexpr double STEP_CYCLES = 100;     // barriers of a step
+// FP32: a round of a block's threads (a pair each, derived and updated) takes
+// its latency, and each warp its issue slots
+constexpr double ROUND_F32 = 900, WARP_F32 = 100;
+// FP64: a warp instruction takes 66 cycles of an SM quarter and 19 of the SM
+constexpr double DERIVE_F64 = 40, UPDATE_F64 = 46;
+
+double f32_cycles(double pairs, int threads, double shared)
+{
+    return STEP_CYCLES + 0.5 * (ROUND_F32 * std::ceil(pairs / threads) + WARP_F32 * shared * std::ceil(pairs / 32));
+}
+double f64_cycles(double nodes, double instructions, double shared)
+{
+    const double warps = shared * std::ceil(nodes / 32);
+    return STEP_CYCLES + instructions * std::max(66.0 * std::ceil(warps / 4), 19.0 * warps);
+}
 
 // nodes that are not solid in [0, x) x [0, y), row length nx + 1
 struct Counts {
@@ -53,7 +69,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
 {
     Plan best;
     int64_t nodes = 0;
-    bool dirichlet = false;
+    bool dirichlet = false, walls = false;
     for (const GridView& g : grids) {
         nodes += (int64_t)g.nx * g.ny;
         for (int y = 0; y < g.ny; ++y)
@@ -68,8 +84,10 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 if (g.edge[ed] == EDGE_PER) return best;  // its inward node may lie outside a window
             }
     }
-    const int64_t limit = f64 ? (int64_t)1 << 19 : (int64_t)1 << 20;
-    if (nodes > limit) return best;
+    if (nodes > (int64_t)1 << 20) return best;
+    for (const GridView& g : grids)
+        for (int y = 0; y < g.ny && !walls; ++y)
+            for (int x = 0; x < g.nx && !walls; ++x) walls = (g.type[(size_t)y * g.pitch + x] & GENERAL_BIT) != 0;
     std::vector<Counts> counts;
     counts.reserve(grids.size());
     for (const GridView& g : grids) counts.emplace_back(g);
@@ -107,38 +125,42 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                     wh = std::max(wh, py ? mh + 2 * k : std::min(g.ny, mh + 2 * k));
                 }
                 Shape s;
-                s.hw = (ww + 5) / 2;
+                s.k = k;
+                s.hw = (ww + 6) / 2;
                 s.rows = wh + 2;
-                s.nlist = s.rows * 2 * s.hw;
-                s.ndir = dirichlet ? 2 * (ww + wh) : 0;
-                const size_t smem = smem_of(per_cell, s);
+                s.ghosts = 2 * (ww + 2) + 2 * wh;
+                s.walls = !f64 && walls ? ww * wh : 0;
+                s.dirs = dirichlet ? 2 * (ww + wh) : 0;
+                const size_t smem = s.cells() * per_cell;
                 if (smem > MAX_SMEM) continue;
                 int np = 1, threads;
                 if (f64) {
-                    threads = std::min(MAX_THREADS, (ww * wh + 31) / 32 * 32);
+                    // (eight warps keep the FP64 pipes busy)
+                    threads = std::min(256, (ww * wh + s.ghosts + 31) / 32 * 32);
+                    s.units = ww * wh;
                 } else {
-                    const int pairs = wh * ((ww + 1) / 2);
-                    np = pairs <= MAX_THREADS ? 1 : pairs <= 2 * MAX_THREADS ? 2 : 4;
-                    if (pairs > MAX_PAIRS * MAX_THREADS) continue;
+                    const int pairs = wh * ((ww + 2) / 2);
+                    np = (pairs + MAX_THREADS - 1) / MAX_THREADS;
+                    if (np > MAX_PAIRS) continue;
                     threads = ((pairs + np - 1) / np + 31) / 32 * 32;
+                    s.units = np * threads;
                 }
-                // blocks of one wave that share an SM, and waves
-                const int fit = std::max(1, std::min((int)(MAX_SMEM / smem), f64 ? 512 / threads : 512 / threads));
+                // blocks of one wave that share an SM (by shared memory and
+                // registers), and waves
+                const int fit = std::max(1, std::min((int)(MAX_SMEM / smem), 65536 / (128 * threads)));
                 const int64_t per_sm = (wet + sms - 1) / sms;
                 const double waves = (double)((per_sm + fit - 1) / fit), shared = (double)std::min<int64_t>(per_sm, fit);
-                double cyc = LAUNCH_CYCLES + LOAD_CELL * ww * wh * shared;
+                double cyc = LOAD_CELL * ww * wh * shared;
+                const double ghosts = (mw >= ww ? 2.0 * wh : 0) + (mh >= wh ? 2.0 * ww : 0);
                 for (int m = k; m >= 1; --m) {
                     // nodes derived and updated with m steps to take
-                    const double cells = 0.5 * (std::min(ww, mw + 2 * m) * (double)std::min(wh, mh + 2 * m) +
-                                                std::min(ww, mw + 2 * m - 2) * (double)std::min(wh, mh + 2 * m - 2));
-                    if (f64) {
-                        const double warps = shared * std::max(1.0, cells / 32);
-                        cyc += STEP_CYCLES + INSTR_F64 * std::max(66.0 * std::min(4.0, warps) / 4, 19.0 * warps);
-                    } else {
-                        cyc += STEP_CYCLES + CELL_F32 * shared * cells;
-                    }
+                    const double da = std::min(ww, mw + 2 * m) * (double)std::min(wh, mh + 2 * m);
+                    const double db = std::min(ww, mw + 2 * m - 2) * (double)std::min(wh, mh + 2 * m - 2);
+                    cyc += f64 ? f64_cycles(da + ghosts, DERIVE_F64, shared) + f64_cycles(db, UPDATE_F64, shared)
+                               : f32_cycles(0.5 * da, threads, shared) + f32_cycles(0.5 * db, threads, shared);
                 }
-                const double cost = waves * cyc / k;
+                // with several blocks on an SM one block's loads hide behind another's steps
+                const double cost = (LAUNCH_CYCLES + (fit > 1 ? BLOCK_CYCLES + waves * cyc : waves * (BLOCK_CYCLES + cyc))) / k;
                 if (cost < best_cost) {
                     best_cost = cost;
                     best.k = k;
@@ -151,7 +173,16 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 }
             }
         }
-    if (best.k == 0) return best;
+    // against one launch per step (us, measured on a GB300): FP32 the row
+    // march, 9.9 us at 512 x 256 nodes, 10.9 at 512 x 512, 13.6 at 1024 x 1024
+    // (a batch's tile kernel 114 for 8 M nodes); FP64 the tile kernel, 29 us
+    // for every full round of the chip's SMs (31 at 512 x 256, 58 at 512 x 512)
+    int64_t tiles64 = 0;
+    for (const GridView& g : grids)
+        tiles64 += (int64_t)((g.nx + tile::TX - 1) / tile::TX) * ((g.ny + tile::TY - 1) / tile::TY);
+    const double single = f64 ? 29.0 * std::max(1.0, std::ceil((double)tiles64 / sms))
+                              : grids.size() > 1 ? 6.0 + nodes / 75e3 : 9.5 + nodes / 220e3;
+    if (best.k == 0 || best_cost / 2070.0 > 0.9 * single) return Plan();
     best.fm = (fmode & F_CORIOLIS) ? 7 : (fmode & F_FRICTION) ? 3 : 1;
     for (size_t i = 0; i < grids.size(); ++i) {
         const GridView& g = grids[i];
@@ -162,6 +193,11 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 if (counts[i](it.x0, it.x1, it.y0, it.y1) > 0) best.items.push_back(it);
             }
     }
+    // At most one tile per SM: ask for more than half an SM's shared memory.
+    // Launches overlap at their ends, and without this the early blocks of the
+    // next one pair up on some SMs while others idle (400 x 3 strip FP64, 4 x 3
+    // tiles: 5.9 us per step, 3.3 with it).
+    if ((int)best.items.size() <= sms) best.smem = std::max(best.smem, MAX_SMEM / 2 + 1024);
     return best;
 }
 
@@ -174,37 +210,80 @@ cudaError_t with_kernel(const Plan& p, F&& f)
     if (p.fm == FMV && p.np == NPV) return f((const void*)step_window_kernel<T, FMV, NPV>);
     MACLAB_W(1, 1) MACLAB_W(3, 1) MACLAB_W(7, 1)
     if constexpr (std::is_same<T, float>::value) {
-        MACLAB_W(1, 2) MACLAB_W(3, 2) MACLAB_W(7, 2) MACLAB_W(1, 4) MACLAB_W(3, 4) MACLAB_W(7, 4)
+        MACLAB_W(1, 2) MACLAB_W(3, 2) MACLAB_W(7, 2) MACLAB_W(1, 3) MACLAB_W(3, 3) MACLAB_W(7, 3) MACLAB_W(1, 4) MACLAB_W(3, 4) MACLAB_W(7, 4)
     }
 #undef MACLAB_W
     return cudaErrorInvalidValue;
 }
 }  // namespace
 
-cudaError_t prepare_launch(const Plan& p, bool f64)
+namespace {
+size_t up(size_t b) { return (b + 255) & ~size_t(255); }
+}  // namespace
+
+size_t list_bytes(const Plan& p)
 {
-    // the kernels are shared by every handle: opt in to the most any plan takes
-    auto opt = [&](const void* k) {
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM);
-    };
-    return f64 ? with_kernel<double>(p, opt) : with_kernel<float>(p, opt);
+    const size_t n = p.items.size();
+    return up(n * sizeof(Item)) + up(n * sizeof(Head)) + up(n * p.shape.units * sizeof(Unit)) +
+           up(n * p.shape.ghosts * sizeof(Ghost)) + up(n * p.shape.walls * 8 * sizeof(Link)) +
+           up(n * p.shape.dirs * sizeof(Dir));
 }
 
 template <typename T>
-cudaError_t launch(const Plan& p, const void* insts, const Item* items, const uint8_t* active, const Buffers<T>& buf,
+cudaError_t build_lists(const Plan& p, const void* insts, void* mem, cudaStream_t stream, Lists* out)
+{
+    const size_t n = p.items.size();
+    unsigned char* q = (unsigned char*)mem;
+    auto take = [&](size_t bytes) {
+        void* r = q;
+        q += up(bytes);
+        return r;
+    };
+    Item* items = (Item*)take(n * sizeof(Item));
+    Head* head = (Head*)take(n * sizeof(Head));
+    Unit* units = (Unit*)take(n * p.shape.units * sizeof(Unit));
+    Ghost* ghosts = (Ghost*)take(n * p.shape.ghosts * sizeof(Ghost));
+    Link* links = (Link*)take(n * p.shape.walls * 8 * sizeof(Link));
+    Dir* dirs = (Dir*)take(n * p.shape.dirs * sizeof(Dir));
+    *out = Lists{head, units, ghosts, links, dirs};
+    cudaError_t e = cudaMemcpyAsync(items, p.items.data(), n * sizeof(Item), cudaMemcpyHostToDevice, stream);
+    // the kernels are shared by every handle: opt in to the most any plan takes
+    if (e == cudaSuccess)
+        e = with_kernel<T>(p, [](const void* k) {
+            return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM);
+        });
+    if (e != cudaSuccess) return e;
+    window_lists_kernel<T><<<(unsigned)n, 256, 0, stream>>>((const BatchInst<T>*)insts, items, p.shape, head, units, ghosts,
+                                                            links, dirs);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch(const Plan& p, const void* insts, const Lists& lists, const uint8_t* active, const Buffers<T>& buf,
                    int steps, const DirTable* tab, cudaStream_t stream)
 {
     static const DirTable none{};
     int steady = tab ? 0 : 1;
-    void* args[] = {(void*)&insts, (void*)&items, (void*)&active, (void*)&buf, (void*)&p.shape,
+    void* args[] = {(void*)&insts, (void*)&lists, (void*)&active, (void*)&buf, (void*)&p.shape,
                     (void*)&steps, (void*)&steady, (void*)(tab ? tab : &none)};
-    return with_kernel<T>(p, [&](const void* k) {
-        return cudaLaunchKernel(k, dim3((unsigned)p.items.size()), dim3((unsigned)p.threads), args, p.smem, stream);
-    });
+    // a launch may begin loading its static data while the one before it ends
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)p.items.size());
+    cfg.blockDim = dim3((unsigned)p.threads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return with_kernel<T>(p, [&](const void* k) { return cudaLaunchKernelExC(&cfg, k, args); });
 }
-template cudaError_t launch<float>(const Plan&, const void*, const Item*, const uint8_t*, const Buffers<float>&, int,
+template cudaError_t build_lists<float>(const Plan&, const void*, void*, cudaStream_t, Lists*);
+template cudaError_t build_lists<double>(const Plan&, const void*, void*, cudaStream_t, Lists*);
+template cudaError_t launch<float>(const Plan&, const void*, const Lists&, const uint8_t*, const Buffers<float>&, int,
                                    const DirTable*, cudaStream_t);
-template cudaError_t launch<double>(const Plan&, const void*, const Item*, const uint8_t*, const Buffers<double>&, int,
+template cudaError_t launch<double>(const Plan&, const void*, const Lists&, const uint8_t*, const Buffers<double>&, int,
                                     const DirTable*, cudaStream_t);
 
 }  // namespace window

@@ -30,13 +30,17 @@ struct Plan {
 // single-step kernels are the better choice).
 Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms);
 
-// Opt in to the plan's shared memory (once per plan).
-cudaError_t prepare_launch(const Plan& p, bool f64);
-
-// `steps` (<= p.k) steps of every tile; insts: BatchInst<T>[], items:
-// p.items on the device; tab: boundary values per step, nullptr when steady.
+// Device memory of a plan's lists, and the lists built there (once per
+// handle; the stream's work must end before p.items goes).  insts: the
+// device's BatchInst<T>[].
+size_t list_bytes(const Plan& p);
 template <typename T>
-cudaError_t launch(const Plan& p, const void* insts, const Item* items, const uint8_t* active, const Buffers<T>& buf,
+cudaError_t build_lists(const Plan& p, const void* insts, void* mem, cudaStream_t stream, Lists* out);
+
+// `steps` (<= p.k) steps of every tile; tab: boundary values per step,
+// nullptr when steady.
+template <typename T>
+cudaError_t launch(const Plan& p, const void* insts, const Lists& lists, const uint8_t* active, const Buffers<T>& buf,
                    int steps, const DirTable* tab, cudaStream_t stream);
 
 }  // namespace window
