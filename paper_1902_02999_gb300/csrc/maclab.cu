@@ -223,6 +223,7 @@ Fields<T> make_fields(const maclab_s* s)
     f.c = make_coef<T>(s->params, s->e, s->dt);
     f.bed = (const T*)s->bed;
     f.bed_plane = (size_t)s->pitch * s->grid.ny;
+    f.boff = 0;
     return f;
 }
 
@@ -1095,6 +1096,7 @@ BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u
         f.c = make_coef<T>(P.params, P.e, P.dt);
         f.bed = bed ? (const T*)bed + o : nullptr;
         f.bed_plane = plane;
+        f.boff = (unsigned)o;
     }
     in.tiles_x = P.tiles_x;
     in.ntiles = P.tiles_x * P.tiles_y;
@@ -2204,6 +2206,8 @@ struct maclab_batch_s {
     unsigned int bar_polls = BARRIER_POLLS;  // polls before a grid-barrier wait gives up
     bool broken = false;            // a persistent step stopped early: the state must be reloaded
     std::vector<uint8_t> reloaded;  // instances set since the batch broke
+    march::BatchGeom mgeom{};       // FP32 row march over the batch (nitems = 0: the tile kernel)
+    int mfm = 0;                    // force terms of any instance
     window::Plan wplan;             // several steps per launch (k = 0: not used)
     window::Lists wlists{};
     void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches, packed
@@ -2341,11 +2345,183 @@ int batch_usable(maclab_batch_t b)
                  "a persistent step stopped early; reload every instance (maclab_batch_set_state) to continue");
 }
 
+// The FP32 row march over every active instance, buffers of parity par.
+cudaError_t batch_march(maclab_batch_t b, int par, cudaStream_t st)
+{
+    Fields<float> f{};
+    f.eta = (const float*)b->eta[par];
+    f.u = (const float*)b->u[par];
+    f.v = (const float*)b->v[par];
+    f.eta1 = (float*)b->eta[1 - par];
+    f.u1 = (float*)b->u[1 - par];
+    f.v1 = (float*)b->v[1 - par];
+    f.D = (const float*)b->D;
+    f.type = b->type;
+    const int blocks = (b->mgeom.nitems + march::WARPS - 1) / march::WARPS;
+    const size_t smem = march::WARPS * sizeof(march::BatchWarpSmem);
+    const BatchInst<float>* insts = (const BatchInst<float>*)b->insts;
+    // absent force terms have zero coefficients and add exact zeros
+    if (b->mfm & F_CORIOLIS)
+        step_march_batch_kernel<7><<<blocks, march::THREADS, smem, st>>>(f, insts, b->active, b->mgeom, par);
+    else
+        step_march_batch_kernel<3><<<blocks, march::THREADS, smem, st>>>(f, insts, b->active, b->mgeom, par);
+    return cudaGetLastError();
+}
+
+// Strip blocks of a batch for the row march: per instance and strip the rows
+// that hold a node that is not solid, cut into tall blocks and short ones,
+// listed tall first as for a single grid (setup_march).  Left to the tile kernel
+// when a Dirichlet node's inward node falls into another strip block (rows:
+// S or N edge) or the packed arrays pass 2^31 elements.
+cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, int sms)
+{
+    if (b->total_np >= (size_t)1 << 31) return cudaSuccess;
+    const size_t smem = march::WARPS * sizeof(march::BatchWarpSmem);
+    int nb = 0;
+    cudaError_t e = cudaSuccess;
+    for (const void* k : {(const void*)step_march_batch_kernel<3>, (const void*)step_march_batch_kernel<7>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, step_march_batch_kernel<3>, march::THREADS, smem);
+    if (e != cudaSuccess) return e;
+    const int resident = std::max(1, nb) * march::WARPS * sms;
+    // strip st of instance i writes columns 60 st - shift .. 60 st + 59 - shift
+    // (shift 2 when the last column would stand alone in a strip, apart from
+    // its neighbour: a Dirichlet node and its inward node stay together)
+    struct Segment {
+        int inst, x0, ya, yb;  // x0: first written column
+    };
+    std::vector<Segment> segs;
+    std::vector<int> first(b->count + 1, 0), shift(b->count, 0);  // segment of strip 0 of each instance
+    std::vector<size_t> at(1, 0);   // first row of each segment in the row tables
+    std::vector<uint8_t> rowflag;   // per segment and row: bit 0 a node that is not solid, bit 1 not plain
+    int64_t rows = 0;
+    for (int i = 0; i < b->count; ++i) {
+        const Prepared& p = P[i];
+        shift[i] = p.nx > 1 && p.nx % march::OUT == 1 ? 2 : 0;
+        const int S = (p.nx - 1 + shift[i]) / march::OUT + 1;
+        first[i] = (int)segs.size();
+        const size_t base = rowflag.size();
+        rowflag.resize(base + (size_t)S * p.ny);
+        for (int y = 0; y < p.ny; ++y) {
+            const uint8_t* t = &p.type[(size_t)y * p.pitch];
+            for (int st = 0; st < S; ++st) {
+                const int x0 = st * march::OUT - shift[i], x1 = std::min(p.nx, x0 + march::OUT);
+                uint8_t any = 0, odd = 0;
+                for (int x = std::max(0, x0); x < x1; ++x) {
+                    any |= t[x] & KIND_MASK;
+                    // fluid and Dirichlet nodes without a bounce-back link are plain
+                    odd |= (uint8_t)(t[x] == MACLAB_SOLID) | (uint8_t)(t[x] == MACLAB_NOSLIP) | (uint8_t)(t[x] & GENERAL_BIT);
+                }
+                rowflag[base + (size_t)st * p.ny + y] = (any ? 1 : 0) | (odd ? 2 : 0);
+            }
+        }
+        for (int st = 0; st < S; ++st) {
+            const uint8_t* fl = &rowflag[base + (size_t)st * p.ny];
+            int ya = 0, yb = p.ny;
+            while (ya < yb && !(fl[ya] & 1)) ++ya;
+            while (yb > ya && !(fl[yb - 1] & 1)) --yb;
+            segs.push_back(Segment{i, st * march::OUT - shift[i], ya, yb});
+            at.push_back(at.back() + p.ny);
+            rows += yb - ya;
+        }
+    }
+    first[b->count] = (int)segs.size();
+    // one wave of tall blocks over 0.9 of the rows, then a third as tall, 16
+    // rows at least: a block reads two more rows than it writes (96 lakes and
+    // channels: 78.5 us; 0.6 and a sixth, 8 rows: 81.4; 1.2: 84.5)
+    constexpr double PHI = 0.9;
+    const int H1 = std::max(16, (int)(PHI * rows / resident)), H2 = std::max(16, H1 / 3);
+    struct Block {
+        int seg, j0, j1;
+    };
+    std::vector<Block> blocks, low;
+    for (int k = 0; k < (int)segs.size(); ++k) {
+        const int len = segs[k].yb - segs[k].ya;
+        int j = segs[k].ya;
+        if (len <= 0) continue;
+        for (int q = (int)(PHI * len / H1 + 0.5); q > 0 && segs[k].yb - j >= H1; --q, j += H1)
+            blocks.push_back(Block{k, j, j + H1});
+        const int rem = segs[k].yb - j, n = (rem + H2 - 1) / H2;
+        for (int q = 0; q < n; ++q)
+            low.push_back(Block{k, j + (int)((int64_t)q * rem / n), j + (int)((int64_t)(q + 1) * rem / n)});
+    }
+    blocks.insert(blocks.end(), low.begin(), low.end());
+    std::vector<int> item_of_row(at.back(), -1);
+    std::vector<int4> items;
+    for (size_t t = 0; t < blocks.size(); ++t) {
+        const Segment& sg = segs[blocks[t].seg];
+        const Prepared& p = P[sg.inst];
+        const int x0 = sg.x0 - 1 - march::HALF, j0 = blocks[t].j0, j1 = blocks[t].j1;
+        bool plain = x0 >= 0 && x0 + 64 <= p.nx && j0 >= 1 && j1 + 1 <= p.ny;
+        for (int j = j0; j < j1; ++j) {
+            item_of_row[at[blocks[t].seg] + j] = (int)t;
+            plain = plain && !(rowflag[at[blocks[t].seg] + j] & 2);
+        }
+        items.push_back(make_int4(sg.inst, x0, j0, j1 | (plain ? 1 << 30 : 0)));
+    }
+    if (items.empty()) return cudaSuccess;
+    auto item_of = [&](int i, int x, int y) {
+        return item_of_row[at[first[i] + (x + shift[i]) / march::OUT] + y];
+    };
+    // Dirichlet nodes per strip block (counting sort by block)
+    const int nstrips = (int)items.size();
+    std::vector<int> ds(nstrips + 1, 0);
+    for (int i = 0; i < b->count; ++i)
+        for (const DirNode& d : P[i].dirs) {
+            const Prepared& p = P[i];
+            const int t = item_of(i, d.x % p.pitch, d.x / p.pitch);
+            if (t != item_of(i, d.n1 % p.pitch, d.n1 / p.pitch) || (p.type[d.n1] & GENERAL_BIT)) return cudaSuccess;
+            ds[t + 1]++;
+        }
+    for (int t = 0; t < nstrips; ++t) ds[t + 1] += ds[t];
+    const bool any_d = ds.back() > 0;
+    std::vector<int> gn, dat(ds);
+    std::vector<DirNode> dn(ds.back());
+    for (int i = 0; i < b->count; ++i) {
+        const Prepared& p = P[i];
+        for (const DirNode& d : p.dirs) dn[dat[item_of(i, d.x % p.pitch, d.x / p.pitch)]++] = d;
+        for (size_t k = 0; k < p.general.size(); k += 32)
+            items.push_back(make_int4(i, -1 - (int)(gn.size() + k), 0, (int)std::min<size_t>(32, p.general.size() - k)));
+        gn.insert(gn.end(), p.general.begin(), p.general.end());
+    }
+    march::BatchGeom g{};
+    auto put = [&](const void* src, size_t bytes) -> void* {
+        void* p = bdev_alloc(b, bytes);
+        if (!p) e = cudaErrorMemoryAllocation;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, b->stream);
+        return p;
+    };
+    g.items = (const int4*)put(items.data(), items.size() * sizeof(int4));
+    if (!gn.empty()) g.glist = (const int*)put(gn.data(), gn.size() * sizeof(int));
+    if (any_d) {
+        g.dstart = (const int*)put(ds.data(), ds.size() * sizeof(int));
+        g.dlist = (const DirNode*)put(dn.data(), dn.size() * sizeof(DirNode));
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return e;
+    g.nitems = (int)items.size();
+    g.nstrips = nstrips;
+    b->mgeom = g;
+    return cudaSuccess;
+}
+
 template <typename T>
 int batch_launch(maclab_batch_t b, cudaStream_t st)
 {
     const int par = b->cur;
     const BatchInst<T>* insts = (const BatchInst<T>*)b->insts;
+    if constexpr (std::is_same<T, float>::value) {
+        if (b->mgeom.nitems > 0) {
+            const cudaError_t e = batch_march(b, par, st);
+            if (e != cudaSuccess)
+                return bfail(b, MACLAB_E_CUDA, std::string("batch step launch: ") + cudaGetErrorString(e));
+            b->cur = 1 - b->cur;
+            b->n += 1;
+            b->have_prev = true;
+            return MACLAB_OK;
+        }
+    }
     // the tiles also update their own nodes with a bounce-back link
     step_batch_kernel<T><<<b->total_tiles, tile::THREADS, tile::smem_bytes<T>(), st>>>(
         insts, b->tile_inst, b->active, par, b->dir_fused ? b->dir_start : nullptr, b->dirs, b->gen_tile_start,
@@ -2649,7 +2825,18 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         }
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        b->mfm = fmode;
         b->wplan = window::make_plan(views, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
+        if (b->prec == MACLAB_F32 && b->wplan.k == 0) {
+            ce = setup_batch_march(b, P, sms > 0 ? sms : 152);
+            if (ce != cudaSuccess) {
+                const int code = ce == cudaErrorMemoryAllocation ? MACLAB_E_NOMEM : MACLAB_E_CUDA;
+                bfail(nullptr, code, std::string("batch row march: ") + cudaGetErrorString(ce));
+                brelease(b);
+                delete b;
+                return code;
+            }
+        }
         if (b->wplan.k > 0) {
             void* mem = bdev_alloc(b, window::list_bytes(b->wplan));
             bool got = mem != nullptr;

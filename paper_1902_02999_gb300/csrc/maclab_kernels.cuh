@@ -82,6 +82,7 @@ struct Fields {
     int idx32;    // 1 when pitch * ny < 2^31: node offsets fit in an int
     int edge[4];  // W, E, S, N
     Coef<T> c;
+    unsigned boff;     // row march over a batch: the instance's first element in the packed arrays
     const T* bed;      // FP64: lambda-weighted stencils of D (sum, x- and y-moment; bed_stencil_kernel),
     size_t bed_plane;  // three planes this many elements apart
 };
@@ -997,7 +998,8 @@ __device__ __forceinline__ void general_node64(const Fields<double>& f, int i, i
              bed_at(f, xi), (f.type[xi] & KIND_MASK) == K_NOSLIP, f.eta1[xi], f.u1[xi], f.v1[xi]);
 }
 
-template <typename T, bool NEW = false>
+// U: links taken at a time (their loads are in flight together).
+template <typename T, bool NEW = false, int U = 1>
 __device__ __forceinline__ void general_node(const Fields<T>& f, int i, int j)
 {
     if constexpr (std::is_same<T, double>::value && !NEW) {
@@ -1011,7 +1013,7 @@ __device__ __forceinline__ void general_node(const Fields<T>& f, int i, int j)
     T Sh = general_rest(c, X);
     T Sx = T(0), Sy = T(0);
     T Q = T(0), Qx = T(0), Qy = T(0);  // new level: sum of lambda G6 (D_x - D_y), weighted by 1, c_x, c_y
-#pragma unroll 1
+#pragma unroll U
     for (int a = 1; a < 9; ++a) {
         const int cx = c_cx[a], cy = c_cy[a];
         const T lam = (a & 1) ? T(1) : T(0.25);

@@ -206,7 +206,9 @@ __device__ __forceinline__ void cp_async_z(uint32_t dst, const void* src, bool v
 // EDGE = true: any strip block; a row outside the grid is resolved
 // through the S / N edge kinds (the same for the whole warp), the lane's
 // columns through its fixed sources; sources behind a wall read zero.
-template <typename T, bool EDGE, typename SM = WarpSmem<T>>
+// B: a batch; the arrays are the packed ones and f.boff is added to every
+// index.
+template <typename T, bool EDGE, typename SM = WarpSmem<T>, bool B = false>
 __device__ __forceinline__ void fetch_row(const Fields<T>& f, int y, int x, const LaneCols2& lc, SM& sm, int slot,
                                           int lane)
 {
@@ -219,7 +221,8 @@ __device__ __forceinline__ void fetch_row(const Fields<T>& f, int y, int x, cons
         rr = resolve_index(y, f.ny, f.edge[2], f.edge[3], 2, fy);
     }
     if (!EDGE || (rr >= 0 && lc.vec)) {
-        const size_t off = EDGE ? (size_t)rr * f.pitch + x : (size_t)(unsigned)(y * f.pitch + x);
+        const size_t off = EDGE ? (size_t)rr * f.pitch + x + (B ? f.boff : 0u)
+                                : (size_t)(unsigned)(y * f.pitch + x + (B ? f.boff : 0u));
 #pragma unroll
         for (int q = 0; q < 4; ++q) cp_async_z<2 * sizeof(T)>(dst + q * FS, fld[q] + off, true);
         // the type bytes of x, x + 1 lie in the aligned word at off & ~3
@@ -227,7 +230,7 @@ __device__ __forceinline__ void fetch_row(const Fields<T>& f, int y, int x, cons
         if constexpr (EDGE) cp_async_z<4>(smem_addr(&sm.rtype[slot][lane][0]), f.type + (off & ~(size_t)3), true);
     } else {
         const bool ok0 = rr >= 0 && lc.c0 >= 0, ok1 = rr >= 0 && lc.c1 >= 0;
-        const size_t row = rr >= 0 ? (size_t)rr * f.pitch : 0;
+        const size_t row = rr >= 0 ? (size_t)rr * f.pitch + (B ? f.boff : 0u) : 0;
         const size_t i0 = ok0 ? row + lc.c0 : 0, i1 = ok1 ? row + lc.c1 : 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -348,7 +351,7 @@ __device__ __forceinline__ void gather_pair(const Coef2& K, float2 A1, float2 M2
 // columns in fcol are a one-node fringe around the strip block; a fringe
 // node is written only if it is a fluid or no-slip node (its own strip
 // block writes a Dirichlet node).
-template <typename T, int FM, bool EDGE, bool FR = false>
+template <typename T, int FM, bool EDGE, bool FR = false, bool B = false>
 __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, const LaneCols2& lc, int last,
                                           unsigned colmask, int lane, WarpSmem<T>& sm, const Coef2& c2, int sp,
                                           int sc, int sm_,
@@ -358,7 +361,7 @@ __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, cons
 {
     using V2 = typename Vec2<T>::type;
     Pair<T> p;
-    if (r + AHEAD <= last) fetch_row<T, EDGE>(f, r + AHEAD, x, lc, sm, sc, lane);
+    if (r + AHEAD <= last) fetch_row<T, EDGE, WarpSmem<T>, B>(f, r + AHEAD, x, lc, sm, sc, lane);
     else asm volatile("cp.async.commit_group;\n" ::);
     asm volatile("cp.async.wait_group %0;\n" ::"n"(AHEAD));
     read_row<T, EDGE>(f, r, x, lc, sm, sp, lane, p);
@@ -416,7 +419,8 @@ __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, cons
                      Eta8{m[1].x, m[2].x, m[3].x, c[1].x, c[3].x, pe[1].x, pe[2].x, pe[3].x}, c[2].x, c[2].y, own.ownh.y,
                      own.hFx.y, own.hFy.y, bed_at(f, ok & 2u ? at + 1 : 0), ns1, oe.y, ou.y, ov.y);
         }
-        const size_t idx = EDGE ? (size_t)(r - 1) * f.pitch + x : (size_t)(unsigned)((r - 1) * f.pitch + x);
+        const size_t idx = EDGE ? (size_t)(r - 1) * f.pitch + x + (B ? f.boff : 0u)
+                                : (size_t)(unsigned)((r - 1) * f.pitch + x + (B ? f.boff : 0u));
         if (!EDGE && OUT == 60) {
             // plain interior block, lanes 0 and 31 pure halo: both columns or none
             if (ok) {
@@ -449,14 +453,14 @@ __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, cons
     }
 }
 
-// Rows j0 .. j1 - 1 of strip s (derived rows j0 - 1 .. j1).  FR: a
+// Rows j0 .. j1 - 1 of the strip from column x0 (derived rows j0 - 1 .. j1).  FR: a
 // fringe pass, which also writes local columns 1 and 62 and whose rows
 // j0 and j1 - 1 are the fringe (see march_row).
-template <typename T, int FM, bool EDGE, bool FR = false>
-__device__ __forceinline__ void march_strip(const Fields<T>& f, const Coef2& c2, int s, int j0, int j1, int lane,
+template <typename T, int FM, bool EDGE, bool FR = false, bool B = false>
+__device__ __forceinline__ void march_strip(const Fields<T>& f, const Coef2& c2, int x0, int j0, int j1, int lane,
                                             WarpSmem<T>& sm)
 {
-    const int x = first_col(s) + 2 * lane;
+    const int x = x0 + 2 * lane;
     // the lane's columns that the strip writes and that lie in the grid
     constexpr int LO = FR ? 1 : 1 + HALF, HI = FR ? 62 : 62 - HALF;
     unsigned colmask = (2 * lane >= LO && 2 * lane <= HI ? 1u : 0u) | (2 * lane + 1 >= LO && 2 * lane + 1 <= HI ? 2u : 0u);
@@ -474,20 +478,20 @@ __device__ __forceinline__ void march_strip(const Fields<T>& f, const Coef2& c2,
     // rows j0 - 1 and j0 in flight in raw slots 0 and 1
 #pragma unroll
     for (int q = 0; q < AHEAD; ++q) {
-        if (j0 - 1 + q <= last) fetch_row<T, EDGE>(f, j0 - 1 + q, x, lc, sm, q, lane);
+        if (j0 - 1 + q <= last) fetch_row<T, EDGE, WarpSmem<T>, B>(f, j0 - 1 + q, x, lc, sm, q, lane);
         else asm volatile("cp.async.commit_group;\n" ::);
     }
     Own<T> own;
     typename Vec2<T>::type o3r[3], edr[3][2];  // carried in registers (CARRY)
     // rows rotate through slots: row r in raw and derived slot (r - j0 + 1) % 3
-    march_row<T, FM, EDGE, FR>(f, j0 - 1, x, lc, last, colmask, lane, sm, c2, 0, 2, 1, own, false, o3r, edr, j0, j1 - 1, fcol);
-    march_row<T, FM, EDGE, FR>(f, j0, x, lc, last, colmask, lane, sm, c2, 1, 0, 2, own, false, o3r, edr, j0, j1 - 1, fcol);
+    march_row<T, FM, EDGE, FR, B>(f, j0 - 1, x, lc, last, colmask, lane, sm, c2, 0, 2, 1, own, false, o3r, edr, j0, j1 - 1, fcol);
+    march_row<T, FM, EDGE, FR, B>(f, j0, x, lc, last, colmask, lane, sm, c2, 1, 0, 2, own, false, o3r, edr, j0, j1 - 1, fcol);
     for (int r = j0 + 1;; r += 3) {
-        march_row<T, FM, EDGE, FR>(f, r, x, lc, last, colmask, lane, sm, c2, 2, 1, 0, own, true, o3r, edr, j0, j1 - 1, fcol);
+        march_row<T, FM, EDGE, FR, B>(f, r, x, lc, last, colmask, lane, sm, c2, 2, 1, 0, own, true, o3r, edr, j0, j1 - 1, fcol);
         if (r >= last) break;
-        march_row<T, FM, EDGE, FR>(f, r + 1, x, lc, last, colmask, lane, sm, c2, 0, 2, 1, own, true, o3r, edr, j0, j1 - 1, fcol);
+        march_row<T, FM, EDGE, FR, B>(f, r + 1, x, lc, last, colmask, lane, sm, c2, 0, 2, 1, own, true, o3r, edr, j0, j1 - 1, fcol);
         if (r + 1 >= last) break;
-        march_row<T, FM, EDGE, FR>(f, r + 2, x, lc, last, colmask, lane, sm, c2, 1, 0, 2, own, true, o3r, edr, j0, j1 - 1, fcol);
+        march_row<T, FM, EDGE, FR, B>(f, r + 2, x, lc, last, colmask, lane, sm, c2, 1, 0, 2, own, true, o3r, edr, j0, j1 - 1, fcol);
         if (r + 2 >= last) break;
     }
     asm volatile("cp.async.wait_group 0;\n" ::);
@@ -657,7 +661,7 @@ step_march_kernel(const __grid_constant__ Fields<T> f, const __grid_constant__ m
     const int item = (int)blockIdx.x * march::WARPS + wib;
     if (item >= g.nitems) return;  // whole warp
     const int4 t = reinterpret_cast<const int4*>(g.items)[item];
-    const int s = t.x, j0 = t.y, j1 = t.z;
+    const int s = march::first_col(t.x), j0 = t.y, j1 = t.z;
     if (t.w) march::march_strip<T, FM, false>(f, march::pairs_of(f.c), s, j0, j1, lane, sm);
     else march::march_strip<T, FM, true>(f, march::pairs_of(f.c), s, j0, j1, lane, sm);
     if (g.gstart) {
@@ -677,9 +681,85 @@ step_march_kernel(const __grid_constant__ Fields<T> f, const __grid_constant__ m
     }
 }
 
-}  // namespace maclab
+// Batched row march (FP32): one launch steps every active instance.  Strip
+// block t (an instance, a strip of its columns, a range of its rows) per
+// warp; the state lies in packed arrays (f's pointers; f.boff and the grid's
+// sizes come from the instance table).  The coefficients differ from warp to
+// warp, so they sit in the warp's shared memory instead of the kernel's
+// parameters (read again each row; in registers they would cost the fifth
+// block of an SM: 120 instead of 96).  96 lakes and channels, 8 M nodes: 78.5
+// us a step against 114 with the tile kernel, whose tiles also compute dry
+// nodes; strips at an instance's W and E edge (two of about five here) take
+// the path with edge rules, which is what keeps it below the 165 G nodes/s of
+// one large grid.
+namespace march {
+struct BatchWarpSmem {
+    WarpSmem<float> s;
+    Coef2 c;
+};
+struct BatchGeom {
+    int nitems;
+    const int4* items;  // a strip block: instance, first derived column, first row, end row | plain << 30;
+                        // nodes with a bounce-back link (up to 32): instance, -1 - first in glist, 0, count
+    const int* glist;
+    const int* dstart;  // as Geom, over the strip blocks
+    const DirNode* dlist;
+    int nstrips;        // items [0, nstrips) are strip blocks
+};
+}  // namespace march
 
-namespace maclab {
+#ifndef MACLAB_MARCH_BATCH_MINB
+#define MACLAB_MARCH_BATCH_MINB 5
+#endif
+template <int FM>
+__global__ void __launch_bounds__(march::THREADS, MACLAB_MARCH_BATCH_MINB)
+step_march_batch_kernel(const __grid_constant__ Fields<float> bases, const BatchInst<float>* __restrict__ insts,
+                        const uint8_t* __restrict__ active, const __grid_constant__ march::BatchGeom g, int parity)
+{
+    extern __shared__ __align__(16) unsigned char march_smem[];
+    const int lane = threadIdx.x & 31, wib = (int)(threadIdx.x >> 5);
+    march::BatchWarpSmem& sm = reinterpret_cast<march::BatchWarpSmem*>(march_smem)[wib];
+    const int item = (int)blockIdx.x * march::WARPS + wib;
+    if (item >= g.nitems) return;  // whole warp
+    const int4 t = g.items[item];
+    if (!active[t.x]) return;
+    const BatchInst<float>& in = insts[t.x];
+    const Fields<float>& fi = in.f[parity];
+    Fields<float> f = bases;
+    f.nx = fi.nx;
+    f.ny = fi.ny;
+    f.pitch = fi.pitch;
+    f.boff = fi.boff;
+    const int s = t.y, j0 = t.z, j1 = t.w & 0x3fffffff;
+    if (item >= g.nstrips) {
+        // nodes with a bounce-back link of one instance, a lane each: small
+        // items of their own at the end of the launch, where they fill warp
+        // slots, instead of a tail of the strip blocks along a shore (which
+        // cost 14 of 93 us on an ensemble of 96 lakes and channels)
+        if (lane < t.w) {
+            const int node = g.glist[-1 - t.y + lane];
+            general_node<float, false, 4>(fi, node % fi.nx, node / fi.nx);
+        }
+        return;
+    }
+    if (lane == 0) sm.c = coef2_of(fi.c);
+    __syncwarp();
+    if (t.w >> 30) {
+        march::march_strip<float, FM, false, false, true>(f, sm.c, s, j0, j1, lane, sm.s);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f.edge[k] = fi.edge[k];
+        march::march_strip<float, FM, true, false, true>(f, sm.c, s, j0, j1, lane, sm.s);
+    }
+    if (g.dstart) {
+        const int b = g.dstart[item], e = g.dstart[item + 1];
+        if (b < e) {
+            __syncwarp();  // the strip block's new values are visible to the warp
+            for (int k = b + lane; k < e; k += 32)
+                dirichlet_node(fi.eta1, fi.u1, fi.v1, fi.D, in.D64, g.dlist[k], in.bv);
+        }
+    }
+}
 
 // Two steps of the strip blocks sel[0 .. n) (plain, see march_strip2) from
 // (eta, u, v) to (eta1, u1, v1).
@@ -714,7 +794,7 @@ step_march_list_kernel(const __grid_constant__ Fields<float> f, const __grid_con
     if (k >= n) return;  // whole warp
     const int item = sel[k];
     const int4 t = reinterpret_cast<const int4*>(g.items)[item];
-    const int s = t.x, j0 = t.y, j1 = t.z;
+    const int s = march::first_col(t.x), j0 = t.y, j1 = t.z;
     if (FR) march::march_strip<float, FM, true, true>(f, march::pairs_of(f.c), s, j0 - 1, j1 + 1, lane, sm);
     else if (t.w) march::march_strip<float, FM, false>(f, march::pairs_of(f.c), s, j0, j1, lane, sm);
     else march::march_strip<float, FM, true>(f, march::pairs_of(f.c), s, j0, j1, lane, sm);

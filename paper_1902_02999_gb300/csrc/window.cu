@@ -38,12 +38,27 @@ double f64_cycles(double nodes, double instructions, double shared)
     return STEP_CYCLES + instructions * std::max(66.0 * std::ceil(warps / 4), 19.0 * warps);
 }
 
-// nodes that are not solid in [0, x) x [0, y), row length nx + 1
+// nodes that are not solid in [0, x) x [0, y), row length nx + 1 (empty when
+// no node is solid), and whether a node has a bounce-back link
 struct Counts {
     std::vector<int> c;
     int w;
-    explicit Counts(const GridView& g) : c((size_t)(g.nx + 1) * (g.ny + 1), 0), w(g.nx + 1)
+    bool walls = false;
+    explicit Counts(const GridView& g) : w(g.nx + 1)
     {
+        bool dry = false;
+        for (int y = 0; y < g.ny; ++y) {
+            const uint8_t* t = g.type + (size_t)y * g.pitch;
+            uint8_t any = 0, solid = 0;
+            for (int x = 0; x < g.nx; ++x) {
+                any |= t[x];
+                solid |= (t[x] & KIND_MASK) == K_SOLID;
+            }
+            walls = walls || (any & GENERAL_BIT);
+            dry = dry || solid;
+        }
+        if (!dry) return;
+        c.assign((size_t)(g.nx + 1) * (g.ny + 1), 0);
         for (int y = 0; y < g.ny; ++y) {
             int run = 0;
             for (int x = 0; x < g.nx; ++x) {
@@ -54,6 +69,7 @@ struct Counts {
     }
     int operator()(int x0, int x1, int y0, int y1) const
     {
+        if (c.empty()) return (x1 - x0) * (y1 - y0);
         return c[(size_t)y1 * w + x1] - c[(size_t)y0 * w + x1] - c[(size_t)y1 * w + x0] + c[(size_t)y0 * w + x0];
     }
 };
@@ -84,15 +100,21 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 if (g.edge[ed] == EDGE_PER) return best;  // its inward node may lie outside a window
             }
     }
-    if (nodes > (int64_t)1 << 20) return best;
-    for (const GridView& g : grids)
-        for (int y = 0; y < g.ny && !walls; ++y)
-            for (int x = 0; x < g.nx && !walls; ++x) walls = (g.type[(size_t)y * g.pitch + x] & GENERAL_BIT) != 0;
+    // (above this the single-step kernels win whatever the tiles)
+    if (nodes > (int64_t)640 << 10) return best;
     std::vector<Counts> counts;
     counts.reserve(grids.size());
-    for (const GridView& g : grids) counts.emplace_back(g);
-    static const int TW[] = {4, 6, 8, 12, 16, 20, 24, 32, 40, 48, 64, 96, 128};
-    static const int TH[] = {2, 3, 4, 6, 8, 12, 16, 20, 24, 32, 40, 48, 64};
+    bool dry = false;
+    for (const GridView& g : grids) {
+        counts.emplace_back(g);
+        walls = walls || counts.back().walls;
+        dry = dry || !counts.back().c.empty();
+    }
+    // without dry nodes to leave out, FP64 gains only where the tile kernel
+    // leaves SMs idle
+    if (f64 && !dry && nodes > (int64_t)140 << 10) return best;
+    static const int TW[] = {4, 8, 12, 16, 24, 32, 40, 48, 64};
+    static const int TH[] = {2, 4, 8, 12, 16, 24, 32, 48};
     static const int KS[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
     const size_t per_cell = f64 ? cell_bytes<double>() : cell_bytes<float>();
     double best_cost = 1e300;
@@ -101,7 +123,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
         for (int th : TH) {
             int64_t upper = 0;
             for (const GridView& g : grids) upper += (int64_t)tiles(g.nx, tw) * tiles(g.ny, th);
-            if (upper > 16 * (int64_t)sms) continue;
+            if (upper > (f64 ? 16 : 4) * (int64_t)sms) continue;
             int64_t wet = 0;
             int mw = 0, mh = 0;
             for (size_t i = 0; i < grids.size(); ++i) {
@@ -109,11 +131,17 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 const int ntx = tiles(g.nx, tw), nty = tiles(g.ny, th);
                 for (int b = 0; b < nty; ++b)
                     for (int a = 0; a < ntx; ++a)
-                        wet += counts[i](cut(g.nx, ntx, a), cut(g.nx, ntx, a + 1), cut(g.ny, nty, b), cut(g.ny, nty, b + 1)) > 0;
+                        wet += counts[i].c.empty() ||
+                               counts[i](cut(g.nx, ntx, a), cut(g.nx, ntx, a + 1), cut(g.ny, nty, b), cut(g.ny, nty, b + 1)) > 0;
                 mw = std::max(mw, (g.nx + ntx - 1) / ntx);
                 mh = std::max(mh, (g.ny + nty - 1) / nty);
             }
             if (wet == 0) continue;
+            // no k can take less than a step of the bare tiles each step
+            const double bare = (double)((wet + sms - 1) / sms) *
+                                (f64 ? 2 * STEP_CYCLES + 19.0 * (DERIVE_F64 + UPDATE_F64) * mw * mh / 32
+                                     : 2 * STEP_CYCLES + WARP_F32 * mw * mh / 64);
+            if (bare >= best_cost) continue;
             for (int k : KS) {
                 if (MACLAB_WINDOW_K > 0 && k != MACLAB_WINDOW_K) continue;
                 // the largest window over the grids
