@@ -107,11 +107,13 @@ __device__ __forceinline__ uint32_t relu2(uint32_t x)
 //   v += res; Y (bf16) and / or Yf (float) [B][R][R][Cout]
 struct ConvArgs {
     const bf16* X;
+    const bf16* XR;   // relu(X) where it is stored (tcgen05 path; read there when relu_in), else nullptr
     const bf16* Wk;
     const float* bias;
     const bf16* gate;
     const bf16* res;
     bf16* Y;
+    bf16* YR;         // relu(Y) stored beside Y (tcgen05 path), or nullptr
     float* Yf;
     int R, Cin, Cout, dil, relu_in;
 };
@@ -461,6 +463,7 @@ __global__ void __launch_bounds__(TC_THREADS) ws_conv_tc_kernel(const ConvArgs a
 struct TmaOperands {
     CUtensorMap A;
     CUtensorMap B;
+    CUtensorMap Y, YR;  // convolution: bf16 output and its rectified copy
 };
 
 // ---------------------------------------------------------------------------
@@ -470,6 +473,7 @@ struct TmaOperands {
 struct WgradArgs {
     const bf16* dY;   // [B][R][R][Cout]
     const bf16* X;    // [B][R][R][Cin]
+    const bf16* XR;   // relu(X) where it is stored, else nullptr
     float* dW;        // [9][Cout][Cin]
     float* part;      // [splits][9][Cout][Cin]: each split's sums, added in order afterwards
     int B, R, Cin, Cout, dil, relu_in, splits;
@@ -871,6 +875,13 @@ __global__ void ws_eta_shift_kernel(int nn, double* h, const uint8_t* mask, cons
     h[k] -= (acc[0] - target) / acc[1];
 }
 
+// relu of bf16 pairs
+__global__ void ws_relu_kernel(const uint32_t* x, uint32_t* y, size_t n)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        y[i] = relu2(x[i]);
+}
+
 int grid_for(size_t n, int cap = 4096) { return (int)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, cap)); }
 
 uint64_t splitmix(uint64_t& s)
@@ -905,6 +916,8 @@ struct maclab_ws_s {
     int64_t step = 0;
     bf16* X = nullptr;          // [B][R][R][16]
     std::vector<bf16*> H;       // H_1 .. H_{L+1}, [B][R][R][C]
+    std::vector<bf16*> HR;      // relu of each that a layer on tcgen05 reads, stored by the layer that writes it; or nullptr
+    int sms = 152;
     bf16* G[2] = {nullptr, nullptr};  // gradient ping-pong [B][R][R][C]
     std::vector<bf16*> GK;      // kept gradients w.r.t. H_1 .. H_{L+1} (maclab_ws_keep_gradients)
     bool keep = false;
@@ -991,17 +1004,12 @@ bool weight_map(CUtensorMap* m, const bf16* Wk, int Cin, int Cout, int bc, int b
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// the tcgen05 kernels' configurations: operand buffers (three stages: two
-// convolution blocks share an SM) and the weight gradient's blocks
-#ifndef MACLAB_T5_CS
-#define MACLAB_T5_CS 1
-#endif
-constexpr int T5_ST = 3, T5_WST = 3;
-// blocks of a cluster sharing each weight stage of the 128 -> 128
-// convolution by multicast (each fetches 1 / T5_CS of it); 1 by default:
-// clusters of 2 and 4 measured slower (forward 0.574 and 0.584 against
-// 0.536 ms), the blocks of a cluster waiting for each other's releases
-constexpr int T5_CS = MACLAB_T5_CS;
+// the tcgen05 kernels' configurations.  A convolution with more tiles than
+// SMs runs two blocks per SM, three stages each (one block's epilogue under
+// the other's main loop); with fewer, one block per SM with six stages, and
+// with at most half as many, 64 output channels a block, so that twice the
+// SMs share the layer.
+constexpr int T5_ST = 3, T5_DEEP = 6, T5_WST = 3;
 constexpr int T5_WBLOCKS = 150;  // weight-gradient blocks: one per SM, 64 KB stages
 template <int KC, int N, int ST>
 constexpr size_t t5_conv_smem()
@@ -1013,19 +1021,21 @@ constexpr size_t t5_wgrad_smem()
 {
     return (size_t)ST * ((MG ? 16384 : N * 128) + 3 * (MG ? N * 128 : 16384)) + 1024;
 }
+template <int KC, int N, int ST, int MINB>
+cudaError_t t5_conv_limit()
+{
+    return cudaFuncSetAttribute(ws_conv5_kernel<KC, N, ST, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)t5_conv_smem<KC, N, ST>());
+}
 
 // set the dynamic shared-memory limit of every tcgen05 kernel instance
 cudaError_t t5_set_limits()
 {
-    cudaError_t e = cudaFuncSetAttribute(ws_conv5_kernel<64, 128, T5_ST, T5_CS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)t5_conv_smem<64, 128, T5_ST>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ws_conv5_kernel<16, 128, T5_ST, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)t5_conv_smem<16, 128, T5_ST>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ws_conv5_kernel<64, 16, T5_ST, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)t5_conv_smem<64, 16, T5_ST>());
+    cudaError_t e = t5_conv_limit<64, 128, T5_ST, 2>();
+    if (e == cudaSuccess) e = t5_conv_limit<64, 128, T5_DEEP, 1>();
+    if (e == cudaSuccess) e = t5_conv_limit<64, 64, T5_DEEP, 1>();
+    if (e == cudaSuccess) e = t5_conv_limit<16, 128, T5_ST, 2>();
+    if (e == cudaSuccess) e = t5_conv_limit<64, 16, T5_DEEP, 1>();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(ws_wgrad5_kernel<true, 128, T5_WST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)t5_wgrad_smem<true, 128, T5_WST>());
@@ -1040,49 +1050,38 @@ cudaError_t t5_set_limits()
 
 // tensor_path 0: the convolution on ws_conv5_kernel; false if its shape or
 // tensor maps are not supported (the caller falls back to mma.sync)
+bool conv5_shape(int R, int Cin, int Cout)
+{
+    return (Cin % 64 == 0 || Cin == 16) && (Cout % 128 == 0 || Cout == 16) && R % 64 == 0 &&
+           (R < 128 ? 128 % R == 0 : R % 128 == 0);
+}
+template <int KC, int N, int ST, int MINB>
+void run_conv5(maclab_ws_t w, const TmaOperands& maps, const ConvArgs& a, int batch)
+{
+    const dim3 grid(batch * (a.R * a.R / 128), a.Cout / N);
+    ws_conv5_kernel<KC, N, ST, MINB><<<grid, T5_THREADS, t5_conv_smem<KC, N, ST>(), w->stream>>>(maps, a, w->tc_err);
+}
 bool launch_conv5(maclab_ws_t w, const ConvArgs& a, int batch)
 {
     const int R = a.R;
-    const bool shape = (a.Cin % 64 == 0 || a.Cin == 16) && (a.Cout % 128 == 0 || a.Cout == 16) && R % 64 == 0 &&
-                       (R < 128 ? 128 % R == 0 : R % 128 == 0);
-    if (!shape) return false;
-    const int KC = a.Cin == 16 ? 16 : 64, N = a.Cout == 16 ? 16 : 128;
+    if (!conv5_shape(R, a.Cin, a.Cout) || (a.relu_in && !a.XR)) return false;
+    if (a.Cin == 16 && a.Cout == 16) return false;  // no such layer
+    const int blocks = batch * (R * R / 128) * std::max(1, a.Cout / 128);
+    const int KC = a.Cin == 16 ? 16 : 64;
+    const int N = a.Cout == 16 ? 16 : KC == 64 && 2 * blocks <= w->sms ? 64 : 128;
     const int bx = R < 128 ? R : 128, by = 128 / bx;
-    const int cs = KC == 64 && N == 128 ? T5_CS : 1;  // the weight box: N / cs rows
     TmaOperands maps;
-    if (!act_map(&maps.A, a.X, a.Cin, R, batch, KC, bx, by) || !weight_map(&maps.B, a.Wk, a.Cin, a.Cout, KC, N / cs))
+    if (!act_map(&maps.A, a.relu_in ? a.XR : a.X, a.Cin, R, batch, KC, bx, by) ||
+        !weight_map(&maps.B, a.Wk, a.Cin, a.Cout, KC, N))
         return false;
-    dim3 grid(batch * (R * R / 128), a.Cout / N);
-    if (KC == 64 && N == 128 && T5_CS == 1) {
-        ws_conv5_kernel<64, 128, T5_ST, 1>
-            <<<grid, T5_THREADS, t5_conv_smem<64, 128, T5_ST>(), w->stream>>>(maps, a, w->tc_err);
-    } else if (KC == 64 && N == 128) {
-        if (grid.x % T5_CS) return false;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(T5_THREADS);
-        cfg.dynamicSmemBytes = t5_conv_smem<64, 128, T5_ST>();
-        cfg.stream = w->stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = T5_CS;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, ws_conv5_kernel<64, 128, T5_ST, T5_CS>, maps, a, w->tc_err) != cudaSuccess) {
-            cudaGetLastError();
-            return false;  // the caller falls back to mma.sync
-        }
-    } else if (KC == 16 && N == 128) {
-        ws_conv5_kernel<16, 128, T5_ST, 1>
-            <<<grid, T5_THREADS, t5_conv_smem<16, 128, T5_ST>(), w->stream>>>(maps, a, w->tc_err);
-    } else if (KC == 64 && N == 16) {
-        ws_conv5_kernel<64, 16, T5_ST, 1>
-            <<<grid, T5_THREADS, t5_conv_smem<64, 16, T5_ST>(), w->stream>>>(maps, a, w->tc_err);
-    } else {
-        return false;  // 16 -> 16 channels: no such layer
-    }
+    if (N != 16 && ((a.Y && !act_map(&maps.Y, a.Y, a.Cout, R, batch, 64, bx, by)) ||
+                    (a.YR && !act_map(&maps.YR, a.YR, a.Cout, R, batch, 64, bx, by))))
+        return false;
+    if (N == 16) run_conv5<64, 16, T5_DEEP, 1>(w, maps, a, batch);
+    else if (KC == 16) run_conv5<16, 128, T5_ST, 2>(w, maps, a, batch);
+    else if (N == 64) run_conv5<64, 64, T5_DEEP, 1>(w, maps, a, batch);
+    else if (blocks <= w->sms) run_conv5<64, 128, T5_DEEP, 1>(w, maps, a, batch);
+    else run_conv5<64, 128, T5_ST, 2>(w, maps, a, batch);
     return true;
 }
 
@@ -1100,6 +1099,10 @@ void launch_conv(maclab_ws_t w, const ConvArgs& a, int batch)
         dim3 grid(batch * a.R * segs, a.Cout / 16);
         ws_conv_kernel<16><<<grid, THREADS, 0, w->stream>>>(a);
     }
+    if (a.YR) {  // a layer that the tcgen05 path could not take still leaves relu(Y) for the next one
+        const size_t n = (size_t)batch * a.R * a.R * a.Cout / 2;
+        ws_relu_kernel<<<grid_for(n), 256, 0, w->stream>>>((const uint32_t*)a.Y, (uint32_t*)a.YR, n);
+    }
 }
 
 // tensor_path 0: the weight gradient on ws_wgrad5_kernel; false if its
@@ -1109,11 +1112,11 @@ bool launch_wgrad5(maclab_ws_t w, const WgradArgs& a0)
     WgradArgs a = a0;
     const bool mg = a.Cout % 128 == 0 && (a.Cin % 128 == 0 || a.Cin == 16);
     const bool head = !mg && a.Cin % 128 == 0 && a.Cout == 16;
-    if (!(mg || head) || a.R % 64) return false;
+    if (!(mg || head) || a.R % 64 || (a.relu_in && !a.XR)) return false;
     const int N = mg ? (a.Cin == 16 ? 16 : 128) : 16;
     const int gbox = (mg || N == 128) ? 64 : 16, xbox = (!mg || N == 128) ? 64 : 16;
     TmaOperands maps;
-    if (!act_map(&maps.A, a.dY, a.Cout, a.R, a.B, gbox, 64, 1) || !act_map(&maps.B, a.X, a.Cin, a.R, a.B, xbox, 64, 1))
+    if (!act_map(&maps.A, a.dY, a.Cout, a.R, a.B, gbox, 64, 1) || !act_map(&maps.B, a.relu_in ? a.XR : a.X, a.Cin, a.R, a.B, xbox, 64, 1))
         return false;
     const int tiles = (mg ? a.Cout / 128 * (a.Cin / N) : a.Cin / 128 * (a.Cout / N));
     const int segs = a.B * a.R * (a.R / 64);
@@ -1186,6 +1189,7 @@ void forward(maclab_ws_t w, int batch)
         const auto& L = w->layers[l];
         ConvArgs a{};
         a.X = in;
+        if (l > 0) a.XR = w->HR[l - 1];
         a.Wk = L.Wf;
         a.bias = w->param + L.b_off;
         a.R = R;
@@ -1197,6 +1201,7 @@ void forward(maclab_ws_t w, int batch)
             a.Yf = w->Yf;
         } else {
             a.Y = w->H[l];
+            a.YR = w->HR[l];
             if (l > 0) a.res = w->H[l - 1];  // residual block
         }
         launch_conv(w, a, batch);
@@ -1221,6 +1226,7 @@ void backward(maclab_ws_t w, int batch)
         WgradArgs g{};
         g.dY = gout;
         g.X = xin;
+        if (l > 0) g.XR = w->HR[l - 1];
         g.dW = w->grad + L.w_off;
         g.B = batch;
         g.R = R;
@@ -1338,7 +1344,18 @@ int maclab_ws_create(const maclab_ws_config* cfg, void* stream, maclab_ws_t* out
     w->part_floats = part_floats_for(w);
     ok = ok && walloc(w, &w->part, w->part_floats) && walloc(w, &w->dpart, 2 * 1024);
     w->H.assign(w->layers.size() - 1, nullptr);
-    for (size_t l = 0; ok && l < w->H.size(); ++l) ok = walloc(w, &w->H[l], P * C);
+    // the tcgen05 path keeps relu(H) beside H (one allocation for both)
+    // where the layer that reads it runs there: every layer, or with channel
+    // counts only the head takes, the last one
+    const bool tc = cfg->tensor_path == 0 && conv5_shape(R, C, IO) && tensor_map_encoder();
+    w->HR.assign(w->H.size(), nullptr);
+    for (size_t l = 0; ok && l < w->H.size(); ++l) {
+        const bool rect = tc && (conv5_shape(R, C, C) || l + 1 == w->H.size());
+        ok = walloc(w, &w->H[l], P * C * (rect ? 2 : 1));
+        if (ok && rect) w->HR[l] = w->H[l] + P * C;
+    }
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev);
     ok = ok && walloc(w, &w->Wf_all, w->nparam) && walloc(w, &w->Wb_all, w->nparam);
     w->table.n = (int)w->layers.size();
     for (int l = 0; ok && l < w->table.n; ++l) {

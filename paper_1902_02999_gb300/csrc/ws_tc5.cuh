@@ -9,13 +9,16 @@
 //   warp 0, lane 0   issues the tensor copies of a stage once the MMAs that
 //                    last read its buffer have completed ("empty");
 //   warp 1, lane 0   issues the stage's MMAs once its operands are in
-//                    ("full", or "ready" after rectification) and commits
-//                    them to the buffer's "empty" barrier;
-//   warps 2..5       rectify the stage's activation operand in shared
-//                    memory when the layer's input is relu(H) (then arrive on
-//                    "ready"), and afterwards read the accumulators out of
-//                    tensor memory (warp w owns lanes 32 (w mod 4) ..) for
-//                    the epilogue.
+//                    ("full") and commits them to the buffer's "empty"
+//                    barrier;
+//   warps 2..5       read the accumulators out of tensor memory afterwards
+//                    (warp w owns lanes 32 (w mod 4) ..) for the epilogue.
+// A layer whose input is relu(H) reads the rectified copy that the layer
+// before stored beside H, so nothing touches a staged operand between its
+// copy and its MMA.  (Rectifying the staged operand instead put 128 threads'
+// pass over 16 to 48 KB, a proxy fence and a barrier into every stage's round
+// trip.  16 samples, forward pass of 14 layers: 0.548 ms, 0.396 without it;
+// training step 1.915 and 1.509 ms; one sample's forward pass 218 and 174 us.)
 // Other lanes of warps 0 and 1 wait at a warp barrier, never spinning on an
 // mbarrier beside the lane that issues.  Every wait is bounded: on time-out
 // the block records it in *err, lets the copies in flight land (bounded)
@@ -86,26 +89,13 @@ __device__ __forceinline__ void t5_load2(uint32_t dst, const CUtensorMap* map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
         : "memory");
 }
-// the same copy delivered to the same offset, and signalled on the same
-// barrier, in every block of the cluster named in mask
-__device__ __forceinline__ void t5_load2_mc(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar,
-                                            uint16_t mask)
+// a box of shared memory to a tensor (bulk group of the issuing thread)
+__device__ __forceinline__ void t5_store4(const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t src)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-        "%3}], [%4], %5;\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar), "h"(mask)
-        : "memory");
-}
-__device__ __forceinline__ uint32_t t5_cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void t5_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(src)
+                 : "memory");
 }
 __device__ __forceinline__ void t5_mma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
 {
@@ -120,28 +110,6 @@ __device__ __forceinline__ void t5_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
                  : "memory");
 }
-// arrives, once the MMAs complete, on the barrier at this offset in every
-// block of the cluster named in mask
-__device__ __forceinline__ void t5_commit_mc(uint32_t bar, uint16_t mask)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::
-                     "r"(bar),
-                 "h"(mask)
-                 : "memory");
-}
-// relu of `bytes` bytes of bf16 pairs, by nt threads (t = 0 .. nt-1)
-__device__ __forceinline__ void t5_rectify(unsigned char* p, uint32_t bytes, int t, int nt)
-{
-    for (uint32_t i = (uint32_t)t * 16u; i < bytes; i += (uint32_t)nt * 16u) {
-        uint4* q = reinterpret_cast<uint4*>(p + i);
-        uint4 v = *q;
-        v.x = relu2(v.x);
-        v.y = relu2(v.y);
-        v.z = relu2(v.z);
-        v.w = relu2(v.w);
-        *q = v;
-    }
-}
 __device__ __forceinline__ void t5_ld16(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(
@@ -154,13 +122,12 @@ __device__ __forceinline__ void t5_ld16(uint32_t taddr, uint32_t (&r)[16])
 }
 
 // Block start-up shared by both kernels: tensor memory (warp 0) and the
-// barriers (thread 0); full and empty count one arrival, ready four (the
-// rectifying warps), done one.
+// barriers (thread 0), one arrival each.
 template <int ST>
 struct T5Bars {
-    uint64_t full[ST], ready[ST], empty[ST], done;
+    uint64_t full[ST], empty[ST], done;
 };
-template <int ST, int CS = 1>
+template <int ST>
 __device__ __forceinline__ uint32_t t5_start(T5Bars<ST>& bars, uint32_t* tmem_slot, uint32_t cols, int* flags)
 {
     const int tid = threadIdx.x;
@@ -173,24 +140,20 @@ __device__ __forceinline__ uint32_t t5_start(T5Bars<ST>& bars, uint32_t* tmem_sl
     if (tid == 0) {
         for (int k = 0; k < ST; ++k) {
             t5_bar_init(smem_addr(&bars.full[k]), 1);
-            t5_bar_init(smem_addr(&bars.ready[k]), 4);
-            t5_bar_init(smem_addr(&bars.empty[k]), CS);  // every block of the cluster releases it
+            t5_bar_init(smem_addr(&bars.empty[k]), 1);
         }
         t5_bar_init(smem_addr(&bars.done), 1);
         flags[0] = flags[1] = flags[2] = 0;  // abort, stages issued, stages seen landed
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    if (CS > 1)
-        t5_cluster_sync();  // no block copies into a peer's buffers before its barriers exist
-    else
-        __syncthreads();
+    __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     return *tmem_slot;
 }
 // Block end: after a time-out, the copies still in flight land (bounded)
 // before shared and tensor memory are released.
-template <int ST, int CS = 1>
+template <int ST>
 __device__ __forceinline__ void t5_finish(T5Bars<ST>& bars, uint32_t tmem, uint32_t cols, int* flags, int* err)
 {
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -199,13 +162,7 @@ __device__ __forceinline__ void t5_finish(T5Bars<ST>& bars, uint32_t tmem, uint3
         for (int s = flags[2]; s < flags[1]; ++s) tc_mbar_wait(smem_addr(&bars.full[s % ST]), (uint32_t)(s / ST) & 1u);
         atomicOr(err, 1);
     }
-    // with a cluster: no block leaves while a peer's copies or MMA
-    // completions may still signal its barriers (every peer has waited for
-    // its own MMAs by now)
-    if (CS > 1)
-        t5_cluster_sync();
-    else
-        __syncthreads();
+    __syncthreads();
     if (threadIdx.x < 32)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(cols) : "memory");
 }
@@ -220,20 +177,24 @@ __device__ __forceinline__ void t5_finish(T5Bars<ST>& bars, uint32_t tmem, uint3
 // outside the image), B = the weights [9 C_out][C_in].  The epilogue warps
 // load the bias into shared memory and their pixel's residual row and gate
 // signs into registers before the main loop, so that only the accumulator
-// is waited for at the end.
+// is waited for at the end.  The bf16 output and its rectified copy go
+// through the stage buffers (free by then, in the swizzle of the tensor
+// map) and out by tensor stores: a thread's own stores would be 16 bytes
+// of a row of 256 each.
 //   stage layout: A chunks [64 / KC] of 128 x KC bf16, then B chunks
 //   [64 / KC] of N x KC bf16, every chunk on a 1024-byte boundary.
-template <int KC, int N, int ST, int CS>
-__global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_constant__ TmaOperands maps,
-                                                               const ConvArgs a, int* err)
+// MINB: blocks per SM; ST stages in flight.
+template <int KC, int N, int ST, int MINB>
+__global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid_constant__ TmaOperands maps,
+                                                                  const ConvArgs a, int* err)
 {
-    constexpr uint16_t MASK = (uint16_t)((1u << CS) - 1u);
     constexpr int CPS = 64 / KC;
     constexpr uint32_t ACH = 128 * KC * 2, BCH = N * KC * 2;
     constexpr uint32_t ABYTES = CPS * ACH, SBYTES = ABYTES + CPS * BCH;
     constexpr uint32_t MODE = KC == 64 ? T5_SW128 : T5_SW32, SBO = KC == 64 ? 1024 : 256;
     constexpr uint32_t IDESC = t5_idesc(128, N, false, false);
     constexpr uint32_t COLS = t5_cols(N);
+    static_assert(N % 64 != 0 || 2 * (N / 64) * 16384u <= ST * SBYTES, "the stores' staging fits the stage buffers");
     extern __shared__ __align__(16) unsigned char t5_raw[];
     __shared__ __align__(8) T5Bars<ST> bars;
     __shared__ uint32_t tmem_slot;
@@ -248,8 +209,7 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
     const int n0 = blockIdx.y * N;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kch = Cin / KC, KT = 9 * kch, NS = (KT + CPS - 1) / CPS;
-    const uint32_t tmem = t5_start<ST, CS>(bars, &tmem_slot, COLS, flags);
-    const int rank = CS > 1 ? (int)t5_cluster_rank() : 0;
+    const uint32_t tmem = t5_start<ST>(bars, &tmem_slot, COLS, flags);
 
     if (warp == 0) {
         if (lane == 0) {
@@ -262,19 +222,12 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
                 }
                 const int c0 = s * CPS, nc = min(CPS, KT - c0);
                 const uint32_t sA = base + buf * SBYTES, sB = sA + ABYTES, bar = smem_addr(&bars.full[buf]);
-                // the block's own A; B whole, of which this block fetches
-                // rows [rank N / CS, (rank + 1) N / CS) for every block of
-                // the cluster (the clusters' blocks share n0)
                 t5_expect(bar, (uint32_t)nc * (ACH + BCH));
                 for (int c = 0; c < nc; ++c) {
                     const int kk = c0 + c, tap = kk / kch, ci0 = (kk % kch) * KC;
                     const int dy = tap / 3 - 1, dx = tap % 3 - 1;
                     t5_load4(sA + c * ACH, &maps.A, ci0, p0 % R + dx * dil, p0 / R + dy * dil, b, bar);
-                    if (CS > 1)
-                        t5_load2_mc(sB + c * BCH + rank * (BCH / CS), &maps.B, ci0, tap * Cout + n0 + rank * (N / CS),
-                                    bar, MASK);
-                    else
-                        t5_load2(sB + c * BCH, &maps.B, ci0, tap * Cout + n0, bar);
+                    t5_load2(sB + c * BCH, &maps.B, ci0, tap * Cout + n0, bar);
                 }
             }
             flags[1] = s;
@@ -285,8 +238,7 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
             int s = 0;
             for (; s < NS; ++s) {
                 const int buf = s % ST;
-                const uint32_t bar = smem_addr(a.relu_in ? &bars.ready[buf] : &bars.full[buf]);
-                if (!tc_mbar_wait(bar, (uint32_t)(s / ST) & 1u)) {
+                if (!tc_mbar_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u)) {
                     atomicOr(&flags[0], 1);
                     break;
                 }
@@ -301,14 +253,9 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
                         t5_mma(tmem, ad, bd, IDESC, (s | c | k16) != 0 ? 1u : 0u);
                     }
                 }
-                // the buffer is free once every block of the cluster is done
-                // with it (its B arrived in all of them together)
-                if (CS > 1)
-                    t5_commit_mc(smem_addr(&bars.empty[buf]), MASK);
-                else
-                    t5_commit(smem_addr(&bars.empty[buf]));
+                t5_commit(smem_addr(&bars.empty[buf]));
             }
-            if (!a.relu_in) flags[2] = s;
+            flags[2] = s;
             // arrives once every MMA issued above has completed
             t5_commit(smem_addr(&bars.done));
         }
@@ -340,30 +287,15 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
             }
         }
         asm volatile("bar.sync 1, 128;\n" ::: "memory");  // sbias written by the four epilogue warps
-        if (a.relu_in) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (!t5_warp_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u, lane)) {
-                    if (lane == 0) atomicOr(&flags[0], 1);
-                    break;
-                }
-                t5_rectify(tsm + buf * SBYTES, ABYTES, tid - 64, T5_THREADS - 64);
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                __syncwarp();
-                if (lane == 0) t5_arrive(smem_addr(&bars.ready[buf]));
-            }
-            if (warp == 2 && lane == 0) flags[2] = s;
-        }
         const bool fin = t5_warp_wait(smem_addr(&bars.done), 0, lane);
         if (!fin && lane == 0) atomicOr(&flags[0], 1);
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        if (fin && !*(volatile int*)&flags[0]) {
+        const bool good = fin && !*(volatile int*)&flags[0];
+        if (good) {
 #pragma unroll
             for (int c0 = 0; c0 < N; c0 += 16) {
                 uint32_t r[16];
                 t5_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                const size_t o = o0 + c0;
                 float v[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -383,23 +315,49 @@ __global__ void __launch_bounds__(T5_THREADS, 2) ws_conv5_kernel(const __grid_co
                     __nv_bfloat162* wb = reinterpret_cast<__nv_bfloat162*>(w2);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) wb[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                    *reinterpret_cast<uint4*>(a.Y + o) = w2[0];
-                    *reinterpret_cast<uint4*>(a.Y + o + 8) = w2[1];
+                    if constexpr (N % 64 == 0) {
+                        // 16-byte chunk c of row m of a half (64 channels) at m 128 + (c ^ m % 8) 16
+                        unsigned char* row = tsm + (c0 / 64) * 16384 + m * 128;
+                        const int ch = (c0 % 64) / 8;
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            uint4* to = reinterpret_cast<uint4*>(row + (((ch + k) ^ (m & 7)) << 4));
+                            *to = w2[k];
+                            if (a.YR)
+                                to[(N / 64) * 1024] = make_uint4(relu2(w2[k].x), relu2(w2[k].y), relu2(w2[k].z), relu2(w2[k].w));
+                        }
+                    } else {
+                        *reinterpret_cast<uint4*>(a.Y + o0 + c0) = w2[0];
+                        *reinterpret_cast<uint4*>(a.Y + o0 + c0 + 8) = w2[1];
+                    }
                 }
                 if (a.Yf) {
 #pragma unroll
                     for (int j = 0; j < 16; j += 4)
-                        *reinterpret_cast<float4*>(a.Yf + o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        *reinterpret_cast<float4*>(a.Yf + o0 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
                 }
             }
         }
+        if constexpr (N % 64 == 0) {
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the staged rows, to the tensor stores
+            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            if (tid == 64 && good && !*(volatile int*)&flags[0] && a.Y) {
+#pragma unroll
+                for (int h = 0; h < N / 64; ++h) {
+                    t5_store4(&maps.Y, n0 + 64 * h, p0 % R, p0 / R, b, base + h * 16384);
+                    if (a.YR) t5_store4(&maps.YR, n0 + 64 * h, p0 % R, p0 / R, b, base + (N / 64 + h) * 16384);
+                }
+                asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;\n" ::: "memory");
+            }
+            __syncwarp();
+        }
     }
-    t5_finish<ST, CS>(bars, tmem, COLS, flags, err);
+    t5_finish<ST>(bars, tmem, COLS, flags, err);
 }
 
 // ---------------------------------------------------------------------------
 // Weight gradient dW[tap][co][ci] = sum_p G[p][co] X[p + d off(tap)][ci]
-// (X = the layer's input, rectified in shared memory when relu_in; G = the
+// (X = the layer's input, the rectified copy where it is relu(H); G = the
 // gradient of its output).  A block owns one row of taps (dy = blockIdx.x
 // - 1, all three dx), a 128-channel tile of one side and an N-channel
 // tile of the other (blockIdx.z), and every 64-pixel row segment of one
@@ -430,7 +388,6 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
     __shared__ int flags[3];
     const uint32_t raw = smem_addr(t5_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    unsigned char* tsm = t5_raw + (base - raw);
     const int R = a.R, Cin = a.Cin, Cout = a.Cout, dil = a.dil;
     const int dy = (int)blockIdx.x - 1, split = blockIdx.y;
     const int mtiles = (MG ? Cout : Cin) / 128;
@@ -483,8 +440,7 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
             int s = 0;
             for (; s < NS; ++s) {
                 const int buf = s % ST;
-                const uint32_t bar = smem_addr(a.relu_in ? &bars.ready[buf] : &bars.full[buf]);
-                if (!tc_mbar_wait(bar, (uint32_t)(s / ST) & 1u)) {
+                if (!tc_mbar_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u)) {
                     atomicOr(&flags[0], 1);
                     break;
                 }
@@ -505,26 +461,11 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
                 }
                 t5_commit(smem_addr(&bars.empty[buf]));
             }
-            if (!a.relu_in) flags[2] = s;
+            flags[2] = s;
             t5_commit(smem_addr(&bars.done));
         }
         __syncwarp();
     } else {
-        if (a.relu_in) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (!t5_warp_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u, lane)) {
-                    if (lane == 0) atomicOr(&flags[0], 1);
-                    break;
-                }
-                t5_rectify(tsm + buf * SBYTES + GSZ, 3 * XSZ, tid - 64, T5_THREADS - 64);
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                __syncwarp();
-                if (lane == 0) t5_arrive(smem_addr(&bars.ready[buf]));
-            }
-            if (warp == 2 && lane == 0) flags[2] = s;
-        }
         const bool fin = t5_warp_wait(smem_addr(&bars.done), 0, lane);
         if (!fin && lane == 0) atomicOr(&flags[0], 1);
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
