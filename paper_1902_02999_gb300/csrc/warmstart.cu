@@ -1055,11 +1055,31 @@ bool conv5_shape(int R, int Cin, int Cout)
     return (Cin % 64 == 0 || Cin == 16) && (Cout % 128 == 0 || Cout == 16) && R % 64 == 0 &&
            (R < 128 ? 128 % R == 0 : R % 128 == 0);
 }
-template <int KC, int N, int ST, int MINB>
-void run_conv5(maclab_ws_t w, const TmaOperands& maps, const ConvArgs& a, int batch)
+// A launch that may begin while the kernel before it ends: its block start-up
+// (barriers, tensor memory) overlaps that kernel's last blocks.  False when
+// the launch failed (the caller falls back to mma.sync).
+template <typename K, typename A>
+bool launch_t5(maclab_ws_t w, K kernel, dim3 grid, size_t smem, const TmaOperands& maps, const A& a)
 {
-    const dim3 grid(batch * (a.R * a.R / 128), a.Cout / N);
-    ws_conv5_kernel<KC, N, ST, MINB><<<grid, T5_THREADS, t5_conv_smem<KC, N, ST>(), w->stream>>>(maps, a, w->tc_err);
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(T5_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = w->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, maps, a, w->tc_err) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+}
+template <int KC, int N, int ST, int MINB>
+bool run_conv5(maclab_ws_t w, const TmaOperands& maps, const ConvArgs& a, int batch)
+{
+    return launch_t5(w, ws_conv5_kernel<KC, N, ST, MINB>, dim3(batch * (a.R * a.R / 128), a.Cout / N),
+                     t5_conv_smem<KC, N, ST>(), maps, a);
 }
 bool launch_conv5(maclab_ws_t w, const ConvArgs& a, int batch)
 {
@@ -1077,12 +1097,11 @@ bool launch_conv5(maclab_ws_t w, const ConvArgs& a, int batch)
     if (N != 16 && ((a.Y && !act_map(&maps.Y, a.Y, a.Cout, R, batch, 64, bx, by)) ||
                     (a.YR && !act_map(&maps.YR, a.YR, a.Cout, R, batch, 64, bx, by))))
         return false;
-    if (N == 16) run_conv5<64, 16, T5_DEEP, 1>(w, maps, a, batch);
-    else if (KC == 16) run_conv5<16, 128, T5_ST, 2>(w, maps, a, batch);
-    else if (N == 64) run_conv5<64, 64, T5_DEEP, 1>(w, maps, a, batch);
-    else if (blocks <= w->sms) run_conv5<64, 128, T5_DEEP, 1>(w, maps, a, batch);
-    else run_conv5<64, 128, T5_ST, 2>(w, maps, a, batch);
-    return true;
+    if (N == 16) return run_conv5<64, 16, T5_DEEP, 1>(w, maps, a, batch);
+    if (KC == 16) return run_conv5<16, 128, T5_ST, 2>(w, maps, a, batch);
+    if (N == 64) return run_conv5<64, 64, T5_DEEP, 1>(w, maps, a, batch);
+    if (blocks <= w->sms) return run_conv5<64, 128, T5_DEEP, 1>(w, maps, a, batch);
+    return run_conv5<64, 128, T5_ST, 2>(w, maps, a, batch);
 }
 
 void launch_conv(maclab_ws_t w, const ConvArgs& a, int batch)
@@ -1123,15 +1142,14 @@ bool launch_wgrad5(maclab_ws_t w, const WgradArgs& a0)
     a.splits = std::max(1, std::min(segs, T5_WBLOCKS / (3 * tiles)));
     a.part = w->part;
     dim3 grid(3, a.splits, tiles);
+    bool ok;
     if (mg && N == 128)
-        ws_wgrad5_kernel<true, 128, T5_WST>
-            <<<grid, T5_THREADS, t5_wgrad_smem<true, 128, T5_WST>(), w->stream>>>(maps, a, w->tc_err);
+        ok = launch_t5(w, ws_wgrad5_kernel<true, 128, T5_WST>, grid, t5_wgrad_smem<true, 128, T5_WST>(), maps, a);
     else if (mg)
-        ws_wgrad5_kernel<true, 16, T5_WST>
-            <<<grid, T5_THREADS, t5_wgrad_smem<true, 16, T5_WST>(), w->stream>>>(maps, a, w->tc_err);
+        ok = launch_t5(w, ws_wgrad5_kernel<true, 16, T5_WST>, grid, t5_wgrad_smem<true, 16, T5_WST>(), maps, a);
     else
-        ws_wgrad5_kernel<false, 16, T5_WST>
-            <<<grid, T5_THREADS, t5_wgrad_smem<false, 16, T5_WST>(), w->stream>>>(maps, a, w->tc_err);
+        ok = launch_t5(w, ws_wgrad5_kernel<false, 16, T5_WST>, grid, t5_wgrad_smem<false, 16, T5_WST>(), maps, a);
+    if (!ok) return false;
     const size_t n = (size_t)9 * a.Cout * a.Cin;
     ws_sum_parts_kernel<<<grid_for(n), 256, 0, w->stream>>>(w->part, a.splits, n, a.dW);
     return true;

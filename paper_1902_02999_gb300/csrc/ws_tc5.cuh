@@ -6,9 +6,9 @@
 //
 // Both kernels split a block's 6 warps by role, each role waiting only on
 // the mbarriers it needs (no block barrier in the main loop):
-//   warp 0, lane 0   issues the tensor copies of a stage once the MMAs that
+//   warp 0           issues the tensor copies of a stage once the MMAs that
 //                    last read its buffer have completed ("empty");
-//   warp 1, lane 0   issues the stage's MMAs once its operands are in
+//   warp 1           issues the stage's MMAs once its operands are in
 //                    ("full") and commits them to the buffer's "empty"
 //                    barrier;
 //   warps 2..5       read the accumulators out of tensor memory afterwards
@@ -19,8 +19,8 @@
 // pass over 16 to 48 KB, a proxy fence and a barrier into every stage's round
 // trip.  16 samples, forward pass of 14 layers: 0.548 ms, 0.396 without it;
 // training step 1.915 and 1.509 ms; one sample's forward pass 218 and 174 us.)
-// Other lanes of warps 0 and 1 wait at a warp barrier, never spinning on an
-// mbarrier beside the lane that issues.  Every wait is bounded: on time-out
+// Warps 0 and 1 run converged, one elected lane issuing (t5_elect).  Every
+// wait is bounded: on time-out
 // the block records it in *err, lets the copies in flight land (bounded)
 // and leaves without writing its outputs.
 
@@ -64,6 +64,25 @@ __device__ __forceinline__ void t5_arrive(uint32_t bar)
 __device__ __forceinline__ void t5_expect(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+// One lane of a converged warp.  The issuing loops run with the whole warp
+// and let this lane issue: the compiler then keeps descriptors and
+// coordinates in uniform registers, which the copies and MMAs take.  Issued
+// from an "if (lane == 0)" they are moved there one by one, about 200 cycles
+// an MMA and a copy, which paced every stage: 790 cycles between the MMAs of
+// one 64-channel stage and the next (clock readings), 345 now.
+__device__ __forceinline__ bool t5_elect()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+// the warp's index, uniform
+__device__ __forceinline__ int t5_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// every lane waits (bounded); the same outcome for the warp
+__device__ __forceinline__ bool t5_wait_all(uint32_t bar, uint32_t parity)
+{
+    return __all_sync(0xffffffffu, tc_mbar_wait(bar, parity)) != 0;
 }
 // lane 0 waits (bounded), the warp learns the outcome
 __device__ __forceinline__ bool t5_warp_wait(uint32_t bar, uint32_t parity, int lane)
@@ -149,6 +168,9 @@ __device__ __forceinline__ uint32_t t5_start(T5Bars<ST>& bars, uint32_t* tmem_sl
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    // launched before the kernel before it ended (launch_t5): everything up
+    // to here touches nothing that one writes
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
     return *tmem_slot;
 }
 // Block end: after a time-out, the copies still in flight land (bounded)
@@ -207,58 +229,86 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
     const int P = R * R, tiles = P / 128;
     const int b = blockIdx.x / tiles, p0 = (blockIdx.x % tiles) * 128;
     const int n0 = blockIdx.y * N;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = t5_warp(), lane = tid & 31;
     const int kch = Cin / KC, KT = 9 * kch, NS = (KT + CPS - 1) / CPS;
     const uint32_t tmem = t5_start<ST>(bars, &tmem_slot, COLS, flags);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (s >= ST && !tc_mbar_wait(smem_addr(&bars.empty[buf]), (uint32_t)(s / ST + 1) & 1u)) {
-                    atomicOr(&flags[0], 1);
+        // running input channel, tap row and column (no divisions on the issue path)
+        int ci0 = 0, tx = 0, row = n0;
+        const int px = p0 % R, py = p0 / R - dil;
+        int x = px - dil, y = py;
+        int s = 0;
+        uint32_t par = 1;
+        bool go = true;
+        while (go && s < NS) {
+#pragma unroll
+            for (int buf = 0; buf < ST; ++buf) {
+                if (s >= NS) break;
+                if (s >= ST && !t5_wait_all(smem_addr(&bars.empty[buf]), par)) {
+                    if (lane == 0) atomicOr(&flags[0], 1);
+                    go = false;
                     break;
                 }
-                const int c0 = s * CPS, nc = min(CPS, KT - c0);
+                const int nc = min(CPS, KT - s * CPS);
                 const uint32_t sA = base + buf * SBYTES, sB = sA + ABYTES, bar = smem_addr(&bars.full[buf]);
-                t5_expect(bar, (uint32_t)nc * (ACH + BCH));
-                for (int c = 0; c < nc; ++c) {
-                    const int kk = c0 + c, tap = kk / kch, ci0 = (kk % kch) * KC;
-                    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                    t5_load4(sA + c * ACH, &maps.A, ci0, p0 % R + dx * dil, p0 / R + dy * dil, b, bar);
-                    t5_load2(sB + c * BCH, &maps.B, ci0, tap * Cout + n0, bar);
+                const bool issue = t5_elect();
+                if (issue) t5_expect(bar, (uint32_t)nc * (ACH + BCH));
+#pragma unroll
+                for (int c = 0; c < CPS; ++c) {
+                    if (c >= nc) break;
+                    if (issue) {
+                        t5_load4(sA + c * ACH, &maps.A, ci0, x, y, b, bar);
+                        t5_load2(sB + c * BCH, &maps.B, ci0, row, bar);
+                    }
+                    ci0 += KC;
+                    if (ci0 == Cin) {
+                        ci0 = 0;
+                        row += Cout;
+                        x += dil;
+                        if (++tx == 3) tx = 0, x = px - dil, y += dil;
+                    }
                 }
+                ++s;
             }
-            flags[1] = s;
+            par ^= 1u;
         }
+        if (lane == 0) flags[1] = s;
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (!tc_mbar_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u)) {
-                    atomicOr(&flags[0], 1);
+        int s = 0;
+        uint32_t par = 0;
+        bool go = true;
+        while (go && s < NS) {
+#pragma unroll
+            for (int buf = 0; buf < ST; ++buf) {
+                if (s >= NS) break;
+                if (!t5_wait_all(smem_addr(&bars.full[buf]), par)) {
+                    if (lane == 0) atomicOr(&flags[0], 1);
+                    go = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const int c0 = s * CPS, nc = min(CPS, KT - c0);
+                const int nc = min(CPS, KT - s * CPS);
                 const uint32_t sA = base + buf * SBYTES, sB = sA + ABYTES;
-                for (int c = 0; c < nc; ++c) {
+                if (t5_elect()) {
 #pragma unroll
-                    for (int k16 = 0; k16 < KC / 16; ++k16) {
-                        const uint64_t ad = t5_desc(sA + c * ACH + k16 * 32, 16, SBO, MODE);
-                        const uint64_t bd = t5_desc(sB + c * BCH + k16 * 32, 16, SBO, MODE);
-                        t5_mma(tmem, ad, bd, IDESC, (s | c | k16) != 0 ? 1u : 0u);
+                    for (int c = 0; c < CPS; ++c) {
+                        if (c >= nc) break;
+                        const uint64_t ad = t5_desc(sA + c * ACH, 16, SBO, MODE), bd = t5_desc(sB + c * BCH, 16, SBO, MODE);
+#pragma unroll
+                        for (int k16 = 0; k16 < KC / 16; ++k16)  // 32 bytes on: 2 in the descriptors' units
+                            t5_mma(tmem, ad + 2 * k16, bd + 2 * k16, IDESC, (buf | c | k16) != 0 || s != 0 ? 1u : 0u);
                     }
+                    t5_commit(smem_addr(&bars.empty[buf]));
                 }
-                t5_commit(smem_addr(&bars.empty[buf]));
+                ++s;
             }
-            flags[2] = s;
-            // arrives once every MMA issued above has completed
-            t5_commit(smem_addr(&bars.done));
+            par ^= 1u;
         }
+        if (lane == 0) flags[2] = s;
+        // arrives once every MMA issued above has completed
+        if (t5_elect()) t5_commit(smem_addr(&bars.done));
         __syncwarp();
     } else {
         // before the main loop: bias to shared memory, this lane's pixel's
@@ -347,7 +397,7 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
                     t5_store4(&maps.Y, n0 + 64 * h, p0 % R, p0 / R, b, base + h * 16384);
                     if (a.YR) t5_store4(&maps.YR, n0 + 64 * h, p0 % R, p0 / R, b, base + (N / 64 + h) * 16384);
                 }
-                asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;\n" ::: "memory");
+                asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
             }
             __syncwarp();
         }
@@ -396,56 +446,55 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
     const int segs_row = R / 64, segs = a.B * R * segs_row;
     const int sg0 = (int)((long long)split * segs / a.splits), sg1 = (int)((long long)(split + 1) * segs / a.splits);
     const int NS = sg1 - sg0;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = t5_warp(), lane = tid & 31;
     const uint32_t tmem = t5_start<ST>(bars, &tmem_slot, COLS, flags);
 
     if (warp == 0) {
-        if (lane == 0) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (s >= ST && !tc_mbar_wait(smem_addr(&bars.empty[buf]), (uint32_t)(s / ST + 1) & 1u)) {
-                    atomicOr(&flags[0], 1);
-                    break;
-                }
-                const int g = sg0 + s, x0 = (g % segs_row) * 64, row = g / segs_row;
-                const int y = row % R, b = row / R;
-                const uint32_t st = base + buf * SBYTES, bar = smem_addr(&bars.full[buf]);
+        // running segment: column block, row, image
+        int x0 = (sg0 % segs_row) * 64, y = (sg0 / segs_row) % R, b = sg0 / segs_row / R;
+        int s = 0, buf = 0;
+        uint32_t par = 1;
+        for (; s < NS; ++s) {
+            if (s >= ST && !t5_wait_all(smem_addr(&bars.empty[buf]), par)) {
+                if (lane == 0) atomicOr(&flags[0], 1);
+                break;
+            }
+            const uint32_t st = base + buf * SBYTES, bar = smem_addr(&bars.full[buf]);
+            if (t5_elect()) {
                 t5_expect(bar, SBYTES);
                 // G tile (maps.A), box of 64 or 16 channels
-                if (GSZ == MSZ) {
-                    t5_load4(st, &maps.A, g0c, x0, y, b, bar);
-                    t5_load4(st + 8192, &maps.A, g0c + 64, x0, y, b, bar);
-                } else {
-                    t5_load4(st, &maps.A, g0c, x0, y, b, bar);
-                }
+                t5_load4(st, &maps.A, g0c, x0, y, b, bar);
+                if (GSZ == MSZ) t5_load4(st + 8192, &maps.A, g0c + 64, x0, y, b, bar);
                 // X tiles of the three taps of this row (maps.B)
 #pragma unroll
                 for (int t = 0; t < 3; ++t) {
                     const uint32_t xt = st + GSZ + t * XSZ;
                     const int xx = x0 + (t - 1) * dil, yy = y + dy * dil;
-                    if (XSZ == MSZ) {
-                        t5_load4(xt, &maps.B, x0c, xx, yy, b, bar);
-                        t5_load4(xt + 8192, &maps.B, x0c + 64, xx, yy, b, bar);
-                    } else {
-                        t5_load4(xt, &maps.B, x0c, xx, yy, b, bar);
-                    }
+                    t5_load4(xt, &maps.B, x0c, xx, yy, b, bar);
+                    if (XSZ == MSZ) t5_load4(xt + 8192, &maps.B, x0c + 64, xx, yy, b, bar);
                 }
             }
-            flags[1] = s;
+            __syncwarp();
+            x0 += 64;
+            if (x0 == R) {
+                x0 = 0;
+                if (++y == R) y = 0, ++b;
+            }
+            if (++buf == ST) buf = 0, par ^= 1u;
         }
+        if (lane == 0) flags[1] = s;
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            int s = 0;
-            for (; s < NS; ++s) {
-                const int buf = s % ST;
-                if (!tc_mbar_wait(smem_addr(&bars.full[buf]), (uint32_t)(s / ST) & 1u)) {
-                    atomicOr(&flags[0], 1);
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t st = base + buf * SBYTES;
+        int s = 0, buf = 0;
+        uint32_t par = 0;
+        for (; s < NS; ++s) {
+            if (!t5_wait_all(smem_addr(&bars.full[buf]), par)) {
+                if (lane == 0) atomicOr(&flags[0], 1);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t st = base + buf * SBYTES;
+            if (t5_elect()) {
 #pragma unroll
                 for (int t = 0; t < 3; ++t) {
                     const uint32_t xt = st + GSZ + t * XSZ;
@@ -461,9 +510,11 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
                 }
                 t5_commit(smem_addr(&bars.empty[buf]));
             }
-            flags[2] = s;
-            t5_commit(smem_addr(&bars.done));
+            __syncwarp();
+            if (++buf == ST) buf = 0, par ^= 1u;
         }
+        if (lane == 0) flags[2] = s;
+        if (t5_elect()) t5_commit(smem_addr(&bars.done));
         __syncwarp();
     } else {
         const bool fin = t5_warp_wait(smem_addr(&bars.done), 0, lane);
