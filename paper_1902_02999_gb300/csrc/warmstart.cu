@@ -723,8 +723,32 @@ constexpr int WS_MAX_LAYERS = 66;
 struct LayerTable {
     int n;
     long long w_off[WS_MAX_LAYERS];
+    long long b_off[WS_MAX_LAYERS];  // bias in the parameter vector
+    long long bpart[WS_MAX_LAYERS];  // bias gradient's block sums
     int cin[WS_MAX_LAYERS], cout[WS_MAX_LAYERS];
 };
+
+// Bias gradients of every layer (block l: layer l) from their block sums, in
+// block order
+__global__ void __launch_bounds__(THREADS) ws_bias_sums_kernel(const float* __restrict__ part,
+                                                               const __grid_constant__ LayerTable tab,
+                                                               float* __restrict__ grad)
+{
+    const int l = blockIdx.x, n = tab.cout[l];
+    const float* p = part + tab.bpart[l];
+    for (int i = threadIdx.x; i < n; i += THREADS) {
+        float t = 0.f;
+        for (int s = 0; s < BG_BLOCKS; s += 16) {
+            float v[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = p[(size_t)(s + j) * n + i];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) t += v[j];
+        }
+        grad[tab.b_off[l] + i] = t;
+    }
+}
+static_assert(BG_BLOCKS % 16 == 0, "sixteen loads are issued before their additions");
 
 // One pass over the parameter vector: with adam, one Adam step (lr_t
 // carries the bias corrections); then every weight is packed in bfloat16
@@ -928,7 +952,8 @@ struct maclab_ws_s {
     float* Yf = nullptr;        // [B][R][R][16]
     double* loss = nullptr;
     double* acc = nullptr;      // decode's (sum of eta, count)
-    float* part = nullptr;      // split and block partial sums of the gradients
+    float* part = nullptr;      // split partial sums of a weight gradient
+    float* bpart = nullptr;     // block partial sums of every layer's bias gradient
     double* dpart = nullptr;    // block partials of the loss and of decode's sums
     size_t part_floats = 0;
     int* tc_err = nullptr;      // set when a tensor-core wait timed out
@@ -987,6 +1012,21 @@ bool act_map(CUtensorMap* m, const bf16* p, int C, int R, int batch, int bc, int
     const cuuint32_t one[4] = {1, 1, 1, 1};
     return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)p, dims, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   bc == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 5-d map [64 channels][x][C / 64][y][batch] of the same tensor: a box of two
+// 64-channel blocks by bx pixels, each block's rows together (128-byte swizzle)
+bool act_map2(CUtensorMap* m, const bf16* p, int C, int R, int batch, int bx)
+{
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)R, (cuuint64_t)(C / 64), (cuuint64_t)R, (cuuint64_t)batch};
+    const cuuint64_t str[4] = {(cuuint64_t)C * 2, 128, (cuuint64_t)R * C * 2, (cuuint64_t)R * R * C * 2};
+    const cuuint32_t box[5] = {64, (cuuint32_t)bx, 2, 1, 1};
+    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)p, dims, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1133,9 +1173,10 @@ bool launch_wgrad5(maclab_ws_t w, const WgradArgs& a0)
     const bool head = !mg && a.Cin % 128 == 0 && a.Cout == 16;
     if (!(mg || head) || a.R % 64 || (a.relu_in && !a.XR)) return false;
     const int N = mg ? (a.Cin == 16 ? 16 : 128) : 16;
-    const int gbox = (mg || N == 128) ? 64 : 16, xbox = (!mg || N == 128) ? 64 : 16;
+    const bf16* x = a.relu_in ? a.XR : a.X;
     TmaOperands maps;
-    if (!act_map(&maps.A, a.dY, a.Cout, a.R, a.B, gbox, 64, 1) || !act_map(&maps.B, a.relu_in ? a.XR : a.X, a.Cin, a.R, a.B, xbox, 64, 1))
+    if (!(mg || N == 128 ? act_map2(&maps.A, a.dY, a.Cout, a.R, a.B, 64) : act_map(&maps.A, a.dY, a.Cout, a.R, a.B, 16, 64, 1)) ||
+        !(!mg || N == 128 ? act_map2(&maps.B, x, a.Cin, a.R, a.B, 64) : act_map(&maps.B, x, a.Cin, a.R, a.B, 16, 64, 1)))
         return false;
     const int tiles = (mg ? a.Cout / 128 * (a.Cin / N) : a.Cin / 128 * (a.Cout / N));
     const int segs = a.B * a.R * (a.R / 64);
@@ -1175,7 +1216,7 @@ void launch_wgrad(maclab_ws_t w, const WgradArgs& a0)
 
 // Floats of the partial-sum buffer: the weight gradient's splits of every
 // layer (at most 304 / (tiles * 9) + 1 of them on mma.sync, T5_WBLOCKS / 3
-// on tcgen05) and the bias gradient's block rows.
+// on tcgen05).
 size_t part_floats_for(const maclab_ws_s* w)
 {
     size_t n = 0;
@@ -1184,7 +1225,6 @@ size_t part_floats_for(const maclab_ws_s* w)
         const int tiles = (L.cout / MT) * (L.cin / NT);
         const size_t S = (size_t)(304 / std::max(1, tiles * 9) + 1);
         n = std::max(n, std::max(S, (size_t)(T5_WBLOCKS / 3)) * 9 * L.cout * L.cin);
-        n = std::max(n, (size_t)BG_BLOCKS * L.cout);
     }
     return n;
 }
@@ -1253,8 +1293,7 @@ void backward(maclab_ws_t w, int batch)
         g.dil = L.dil;
         g.relu_in = L.relu_in;
         launch_wgrad(w, g);
-        ws_bias_grad_kernel<<<BG_BLOCKS, THREADS, 0, w->stream>>>(gout, P, L.cout, w->part);
-        ws_sum_parts_kernel<<<grid_for(L.cout), 256, 0, w->stream>>>(w->part, BG_BLOCKS, L.cout, w->grad + L.b_off);
+        ws_bias_grad_kernel<<<BG_BLOCKS, THREADS, 0, w->stream>>>(gout, P, L.cout, w->bpart + w->table.bpart[l]);
         if (l == 0) break;
         // gradient w.r.t. this layer's input H_{l-1}:
         //   head:  relu'(H) * conv^T(gout)
@@ -1274,6 +1313,9 @@ void backward(maclab_ws_t w, int batch)
         gout = a.Y;
         ping ^= 1;
     }
+    // every layer's block sums at once: one layer's are a chain of BG_BLOCKS
+    // additions per channel on one block, 10 us of an idle chip each
+    ws_bias_sums_kernel<<<nl, THREADS, 0, w->stream>>>(w->bpart, w->table, w->grad);
     w->grad_batch = w->keep ? batch : 0;
 }
 
@@ -1360,7 +1402,9 @@ int maclab_ws_create(const maclab_ws_config* cfg, void* stream, maclab_ws_t* out
               walloc(w, &w->Yf, P * IO) && walloc(w, &w->loss, 1) && walloc(w, &w->acc, 2) && walloc(w, &w->tc_err, 1) && walloc(w, &w->G[0], P * C) &&
               walloc(w, &w->G[1], P * C);
     w->part_floats = part_floats_for(w);
-    ok = ok && walloc(w, &w->part, w->part_floats) && walloc(w, &w->dpart, 2 * 1024);
+    size_t biases = 0;
+    for (const auto& L : w->layers) biases += L.cout;
+    ok = ok && walloc(w, &w->bpart, BG_BLOCKS * biases) && walloc(w, &w->part, w->part_floats) && walloc(w, &w->dpart, 2 * 1024);
     w->H.assign(w->layers.size() - 1, nullptr);
     // the tcgen05 path keeps relu(H) beside H (one allocation for both)
     // where the layer that reads it runs there: every layer, or with channel
@@ -1381,6 +1425,8 @@ int maclab_ws_create(const maclab_ws_config* cfg, void* stream, maclab_ws_t* out
         L.Wf = w->Wf_all + L.w_off;
         L.Wb = w->Wb_all + L.w_off;
         w->table.w_off[l] = L.w_off;
+        w->table.b_off[l] = L.b_off;
+        w->table.bpart[l] = l ? w->table.bpart[l - 1] + (long long)BG_BLOCKS * w->layers[l - 1].cout : 0;
         w->table.cin[l] = L.cin;
         w->table.cout[l] = L.cout;
     }

@@ -100,6 +100,15 @@ __device__ __forceinline__ void t5_load4(uint32_t dst, const CUtensorMap* map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
 }
+// [64 channels][x][channel block][y][image]: a box of several channel blocks
+__device__ __forceinline__ void t5_load5(uint32_t dst, const CUtensorMap* map, int x, int block, int y, int b, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
+        "[%7];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(x), "r"(block), "r"(y), "r"(b), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void t5_load2(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar)
 {
     asm volatile(
@@ -128,6 +137,18 @@ __device__ __forceinline__ void t5_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
                  : "memory");
+}
+__device__ __forceinline__ void t5_ld32(uint32_t taddr, uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ void t5_ld16(uint32_t taddr, uint32_t (&r)[16])
 {
@@ -168,10 +189,16 @@ __device__ __forceinline__ uint32_t t5_start(T5Bars<ST>& bars, uint32_t* tmem_sl
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    // launched before the kernel before it ended (launch_t5): everything up
-    // to here touches nothing that one writes
-    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     return *tmem_slot;
+}
+// The block may have started before the kernel before it ended (launch_t5):
+// waits until that one's results are there.  Weights and biases, written only
+// by kernels that let no later one start early, may be read before.
+__device__ __forceinline__ void t5_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void t5_prefetch(const CUtensorMap* map)
+{
+    asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 // Block end: after a time-out, the copies still in flight land (bounded)
 // before shared and tensor memory are released.
@@ -231,21 +258,68 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
     const int n0 = blockIdx.y * N;
     const int tid = threadIdx.x, warp = t5_warp(), lane = tid & 31;
     const int kch = Cin / KC, KT = 9 * kch, NS = (KT + CPS - 1) / CPS;
+    if (tid == 32) {
+        t5_prefetch(&maps.A);
+        t5_prefetch(&maps.B);
+    }
     const uint32_t tmem = t5_start<ST>(bars, &tmem_slot, COLS, flags);
 
     if (warp == 0) {
-        // running input channel, tap row and column (no divisions on the issue path)
-        int ci0 = 0, tx = 0, row = n0;
-        const int px = p0 % R, py = p0 / R - dil;
-        int x = px - dil, y = py;
-        int s = 0;
-        uint32_t par = 1;
+        // running weight row and, for A, tap column and position (no
+        // divisions on the issue path)
+        int cb = 0, row = n0;
+        auto next_b = [&] {
+            cb += KC;
+            if (cb == Cin) cb = 0, row += Cout;
+        };
+        const int px = p0 % R;
+        int ci0 = 0, tx = 0, x = px - dil, y = p0 / R - dil;
+        auto next_a = [&] {
+            ci0 += KC;
+            if (ci0 == Cin) {
+                ci0 = 0;
+                x += dil;
+                if (++tx == 3) tx = 0, x = px - dil, y += dil;
+            }
+        };
+        // the first stages: weights before the kernel before this one has
+        // ended, activations after
+#pragma unroll
+        for (int buf = 0; buf < ST; ++buf) {
+            if (buf >= NS) break;
+            const int nc = min(CPS, KT - buf * CPS);
+            const uint32_t sB = base + buf * SBYTES + ABYTES, bar = smem_addr(&bars.full[buf]);
+            const bool issue = t5_elect();
+            if (issue) t5_expect(bar, (uint32_t)nc * (ACH + BCH));
+#pragma unroll
+            for (int c = 0; c < CPS; ++c) {
+                if (c >= nc) break;
+                if (issue) t5_load2(sB + c * BCH, &maps.B, cb, row, bar);
+                next_b();
+            }
+        }
+        t5_dep_wait();
+#pragma unroll
+        for (int buf = 0; buf < ST; ++buf) {
+            if (buf >= NS) break;
+            const int nc = min(CPS, KT - buf * CPS);
+            const uint32_t sA = base + buf * SBYTES, bar = smem_addr(&bars.full[buf]);
+            const bool issue = t5_elect();
+#pragma unroll
+            for (int c = 0; c < CPS; ++c) {
+                if (c >= nc) break;
+                if (issue) t5_load4(sA + c * ACH, &maps.A, ci0, x, y, b, bar);
+                next_a();
+            }
+        }
+        int s = min(ST, NS);
+        uint32_t par = 0;
         bool go = true;
         while (go && s < NS) {
 #pragma unroll
             for (int buf = 0; buf < ST; ++buf) {
                 if (s >= NS) break;
-                if (s >= ST && !t5_wait_all(smem_addr(&bars.empty[buf]), par)) {
+                if (!t5_wait_all(smem_addr(&bars.empty[buf]), par)) {
                     if (lane == 0) atomicOr(&flags[0], 1);
                     go = false;
                     break;
@@ -259,15 +333,10 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
                     if (c >= nc) break;
                     if (issue) {
                         t5_load4(sA + c * ACH, &maps.A, ci0, x, y, b, bar);
-                        t5_load2(sB + c * BCH, &maps.B, ci0, row, bar);
+                        t5_load2(sB + c * BCH, &maps.B, cb, row, bar);
                     }
-                    ci0 += KC;
-                    if (ci0 == Cin) {
-                        ci0 = 0;
-                        row += Cout;
-                        x += dil;
-                        if (++tx == 3) tx = 0, x = px - dil, y += dil;
-                    }
+                    next_a();
+                    next_b();
                 }
                 ++s;
             }
@@ -317,6 +386,7 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
         const int m = q * 32 + lane;
         const size_t o0 = ((size_t)b * P + p0 + m) * Cout + n0;
         for (int c = tid - 64; c < N; c += T5_THREADS - 64) sbias[c] = a.bias ? a.bias[n0 + c] : 0.f;
+        t5_dep_wait();
         uint4 rres[N / 8];
         uint32_t gbits[(N + 31) / 32];
 #pragma unroll
@@ -341,65 +411,73 @@ __global__ void __launch_bounds__(T5_THREADS, MINB) ws_conv5_kernel(const __grid
         if (!fin && lane == 0) atomicOr(&flags[0], 1);
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const bool good = fin && !*(volatile int*)&flags[0];
-        if (good) {
+        constexpr int CW = N % 32 == 0 ? 32 : 16;  // columns read from tensor memory at a time
+        constexpr int HW = N % 64 == 0 ? 64 : N;   // columns of one output box
 #pragma unroll
-            for (int c0 = 0; c0 < N; c0 += 16) {
-                uint32_t r[16];
-                t5_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-                float v[16];
+        for (int h0 = 0; h0 < N; h0 += HW) {
+            if (good) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    v[j] = __uint_as_float(r[j]) + sbias[c0 + j];
-                    if (!((gbits[(c0 + j) >> 5] >> ((c0 + j) & 31)) & 1u)) v[j] = 0.f;
-                }
-                if (a.res) {
-                    const __nv_bfloat162* rr = reinterpret_cast<const __nv_bfloat162*>(&rres[c0 / 8]);
+                for (int c0 = h0; c0 < h0 + HW; c0 += CW) {
+                    uint32_t r[CW];
+                    const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+                    if constexpr (CW == 32) t5_ld32(ta, r);
+                    else t5_ld16(ta, r);
+                    float v[CW];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        v[2 * j] += __bfloat162float(rr[j].x);
-                        v[2 * j + 1] += __bfloat162float(rr[j].y);
+                    for (int j = 0; j < CW; ++j) {
+                        v[j] = __uint_as_float(r[j]) + sbias[c0 + j];
+                        if (!((gbits[(c0 + j) >> 5] >> ((c0 + j) & 31)) & 1u)) v[j] = 0.f;
                     }
-                }
-                if (a.Y) {
-                    uint4 w2[2];
-                    __nv_bfloat162* wb = reinterpret_cast<__nv_bfloat162*>(w2);
+                    if (a.res) {
+                        const __nv_bfloat162* rr = reinterpret_cast<const __nv_bfloat162*>(&rres[c0 / 8]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) wb[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                    if constexpr (N % 64 == 0) {
-                        // 16-byte chunk c of row m of a half (64 channels) at m 128 + (c ^ m % 8) 16
-                        unsigned char* row = tsm + (c0 / 64) * 16384 + m * 128;
-                        const int ch = (c0 % 64) / 8;
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            uint4* to = reinterpret_cast<uint4*>(row + (((ch + k) ^ (m & 7)) << 4));
-                            *to = w2[k];
-                            if (a.YR)
-                                to[(N / 64) * 1024] = make_uint4(relu2(w2[k].x), relu2(w2[k].y), relu2(w2[k].z), relu2(w2[k].w));
+                        for (int j = 0; j < CW / 2; ++j) {
+                            v[2 * j] += __bfloat162float(rr[j].x);
+                            v[2 * j + 1] += __bfloat162float(rr[j].y);
                         }
-                    } else {
-                        *reinterpret_cast<uint4*>(a.Y + o0 + c0) = w2[0];
-                        *reinterpret_cast<uint4*>(a.Y + o0 + c0 + 8) = w2[1];
+                    }
+                    if (a.Y) {
+#pragma unroll
+                        for (int k = 0; k < CW / 8; ++k) {
+                            uint4 w2;
+                            __nv_bfloat162* wb = reinterpret_cast<__nv_bfloat162*>(&w2);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) wb[j] = __floats2bfloat162_rn(v[8 * k + 2 * j], v[8 * k + 2 * j + 1]);
+                            if constexpr (N % 64 == 0) {
+                                // 16-byte chunk c of row m of a box (64 channels) at m 128 + (c ^ m % 8) 16
+                                const int ch = (c0 - h0) / 8 + k;
+                                uint4* to = reinterpret_cast<uint4*>(tsm + (h0 / 64) * 16384 + m * 128 + ((ch ^ (m & 7)) << 4));
+                                *to = w2;
+                                if (a.YR) to[(N / 64) * 1024] = make_uint4(relu2(w2.x), relu2(w2.y), relu2(w2.z), relu2(w2.w));
+                            } else {
+                                *reinterpret_cast<uint4*>(a.Y + o0 + c0 + 8 * k) = w2;
+                            }
+                        }
+                    }
+                    if (a.Yf) {
+#pragma unroll
+                        for (int j = 0; j < CW; j += 4)
+                            *reinterpret_cast<float4*>(a.Yf + o0 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
                     }
                 }
-                if (a.Yf) {
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4)
-                        *reinterpret_cast<float4*>(a.Yf + o0 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+            if constexpr (N % 64 == 0) {
+                // one box is on its way while the next is computed
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the staged rows, to the tensor stores
+                asm volatile("bar.sync 1, 128;\n" ::: "memory");
+                if (warp == 2 && good && !*(volatile int*)&flags[0] && a.Y) {
+                    if (t5_elect()) {
+                        t5_store4(&maps.Y, n0 + h0, p0 % R, p0 / R, b, base + (h0 / 64) * 16384);
+                        if (a.YR) t5_store4(&maps.YR, n0 + h0, p0 % R, p0 / R, b, base + (N / 64 + h0 / 64) * 16384);
+                        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                    }
+                    __syncwarp();
                 }
             }
         }
         if constexpr (N % 64 == 0) {
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the staged rows, to the tensor stores
-            asm volatile("bar.sync 1, 128;\n" ::: "memory");
-            if (tid == 64 && good && !*(volatile int*)&flags[0] && a.Y) {
-#pragma unroll
-                for (int h = 0; h < N / 64; ++h) {
-                    t5_store4(&maps.Y, n0 + 64 * h, p0 % R, p0 / R, b, base + h * 16384);
-                    if (a.YR) t5_store4(&maps.YR, n0 + 64 * h, p0 % R, p0 / R, b, base + (N / 64 + h) * 16384);
-                }
-                asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
-            }
-            __syncwarp();
+            // shared memory is read before the block leaves (a lane without stores passes at once)
+            if (warp == 2) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
         }
     }
     t5_finish<ST>(bars, tmem, COLS, flags, err);
@@ -447,7 +525,12 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
     const int sg0 = (int)((long long)split * segs / a.splits), sg1 = (int)((long long)(split + 1) * segs / a.splits);
     const int NS = sg1 - sg0;
     const int tid = threadIdx.x, warp = t5_warp(), lane = tid & 31;
+    if (tid == 32) {
+        t5_prefetch(&maps.A);
+        t5_prefetch(&maps.B);
+    }
     const uint32_t tmem = t5_start<ST>(bars, &tmem_slot, COLS, flags);
+    t5_dep_wait();
 
     if (warp == 0) {
         // running segment: column block, row, image
@@ -462,16 +545,16 @@ __global__ void __launch_bounds__(T5_THREADS) ws_wgrad5_kernel(const __grid_cons
             const uint32_t st = base + buf * SBYTES, bar = smem_addr(&bars.full[buf]);
             if (t5_elect()) {
                 t5_expect(bar, SBYTES);
-                // G tile (maps.A), box of 64 or 16 channels
-                t5_load4(st, &maps.A, g0c, x0, y, b, bar);
-                if (GSZ == MSZ) t5_load4(st + 8192, &maps.A, g0c + 64, x0, y, b, bar);
+                // G tile (maps.A): two boxes of 64 channels in one copy, or 16 channels
+                if (GSZ == MSZ) t5_load5(st, &maps.A, x0, g0c / 64, y, b, bar);
+                else t5_load4(st, &maps.A, g0c, x0, y, b, bar);
                 // X tiles of the three taps of this row (maps.B)
 #pragma unroll
                 for (int t = 0; t < 3; ++t) {
                     const uint32_t xt = st + GSZ + t * XSZ;
                     const int xx = x0 + (t - 1) * dil, yy = y + dy * dil;
-                    t5_load4(xt, &maps.B, x0c, xx, yy, b, bar);
-                    if (XSZ == MSZ) t5_load4(xt + 8192, &maps.B, x0c + 64, xx, yy, b, bar);
+                    if (XSZ == MSZ) t5_load5(xt, &maps.B, xx, x0c / 64, yy, b, bar);
+                    else t5_load4(xt, &maps.B, x0c, xx, yy, b, bar);
                 }
             }
             __syncwarp();
