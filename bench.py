@@ -36,9 +36,9 @@ METRIC = ("MLUPS & % of HBM roofline (FP32 step); wall time to residual 1e-8, "
 BYTES_PER_NODE = {"f32": 29, "f64": 57}   # read eta,u,v,D + type, write eta,u,v
 HBM_NOMINAL_GBS = 7900.0                   # GB300 HBM3e, nominal
 # FP64 arithmetic of one node update, multiply-add counted as two: the
-# source quantities (53, with the friction term) and the gather / update (67),
+# source quantities (44, with the friction term) and the gather / update (58),
 # plus one square root and one reciprocal
-F64_FLOPS_PER_NODE = 120
+F64_FLOPS_PER_NODE = 102
 F64_NOMINAL_TFLOPS = 1.25                  # GB300 dense FP64, nominal (the bench also measures it)
 FALLBACK_HBM_GBS = 6800.0
 FALLBACK_BF16_TFLOPS = 1900.0
