@@ -1115,11 +1115,14 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     const bool f64 = s->prec == MACLAB_F64;
     s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0}}, f64, s->fmode, sms);
     if (s->wplan.k == 0) return MACLAB_OK;
-    const size_t NP = (size_t)P.pitch * P.ny;
-    void* mem = dev_alloc(s, window::list_bytes(s->wplan));
-    bool ok = mem != nullptr && (s->winst = dev_alloc(s, f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>))) != nullptr;
-    for (int q = 0; q < 3 && ok; ++q) ok = (s->wmid[q] = dev_alloc(s, NP * s->esize)) != nullptr;
-    if (!ok) return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
+    // one allocation: lists, instance table, scratch state
+    const auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
+    const size_t NP = (size_t)P.pitch * P.ny, state = up(NP * s->esize), lists = up(window::list_bytes(s->wplan));
+    const size_t inst = up(f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>));
+    unsigned char* mem = (unsigned char*)dev_alloc(s, lists + inst + 3 * state);
+    if (!mem) return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
+    s->winst = mem + lists;
+    for (int q = 0; q < 3; ++q) s->wmid[q] = mem + lists + inst + q * state;
     cudaError_t e = cudaSuccess;
     BatchInst<float> f{};
     BatchInst<double> d{};
