@@ -94,11 +94,11 @@ class _TorchAllocator:
 
 
 class _DeviceArray:
-    """Device memory in the form torch.as_tensor takes."""
+    """Device memory in the form torch.as_tensor takes (strides in bytes)."""
 
-    def __init__(self, ptr: int, shape, typestr: str):
+    def __init__(self, ptr: int, shape, strides, typestr: str):
         self.__cuda_array_interface__ = {"shape": shape, "typestr": typestr, "data": (ptr, False), "version": 3,
-                                         "strides": None}
+                                         "strides": strides}
 
 
 _live = weakref.WeakSet()
@@ -177,7 +177,6 @@ class Simulation:
         self._check(self._lib.maclab_get_info(self._h, ctypes.byref(info)))
         self.info = {f: getattr(info, f) for f, _ in _abi.Info._fields_}
         self.precision = "f32" if prec == F32 else "f64"
-        self._views = {}
 
     # -- construction from an ``inputs.Case``-like object ---------------------
     @classmethod
@@ -315,21 +314,22 @@ class Simulation:
         return float(t.value), int(n.value)
 
     def device_state(self):
-        """Zero-copy torch views (ny, nx) of the current device state (eta, u, v)."""
+        """Zero-copy torch views (ny, nx) of the current device state (eta, u, v).
+
+        New tensors on every call: one that was kept would carry the modes of
+        the call that made it (an inference tensor for good) and its autograd
+        history into later ones.  They name the handle's GPU, since under
+        another current device torch would copy the state there.  (Three
+        views with their strides take 6 us; slicing the padded arrays 19 us,
+        slicing kept tensors 9 us.)
+        """
+        import torch
         ptrs = [ctypes.c_void_p() for _ in range(3)]
         self._check(self._lib.maclab_device_state(self._h, *[ctypes.byref(p) for p in ptrs]))
-        return tuple(self._view(p.value)[:, :self.nx] for p in ptrs)
-
-    def _view(self, ptr: int):
-        """The padded array at one of the handle's own state buffers, which
-        stay where they are for its lifetime (six views in all: building one
-        costs about 8 us, a third of a short call's time)."""
-        view = self._views.get(ptr)
-        if view is None:
-            import torch
-            array = _DeviceArray(ptr, (self.ny, self.info["pitch"]), "<f4" if self.precision == "f32" else "<f8")
-            view = self._views[ptr] = torch.as_tensor(array, device="cuda")
-        return view
+        size, typestr = (4, "<f4") if self.precision == "f32" else (8, "<f8")
+        shape, strides = (self.ny, self.nx), (self.info["pitch"] * size, size)
+        device = torch.device("cuda", self.device)
+        return tuple(torch.as_tensor(_DeviceArray(p.value, shape, strides, typestr), device=device) for p in ptrs)
 
     def close(self) -> None:
         if getattr(self, "_h", None):
