@@ -143,31 +143,12 @@ template <> struct Op<double> {
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-    // An FP64 warp instruction holds its SM quarter's pipe for 64 cycles, so
-    // these are written for few of them: the hardware's approximation (about
-    // 20 bits; it takes no FP64 slot) and one third-order step, which leaves
-    // an error of about an ulp.  With r = 1 - a y the reciprocal is
-    // y / (1 - r) = y (1 + r + r^2 + ...); with r = 1 - a y^2 the root is
-    // a y (1 - r)^(-1/2) = a y (1 + r / 2 + 3 r^2 / 8 + ...).
-    static __device__ __forceinline__ double rcp(double a)
-    {
-        const unsigned ex = (unsigned)__double2hiint(a) & 0x7fffffffu;
-        if (ex - 0x00200000u >= 0x7fa00000u) return 1.0 / a;  // zero, subnormal, huge, inf, nan (or their reciprocal)
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-        const double r = __fma_rn(-a, y, 1.0);
-        return __fma_rn(y, __fma_rn(r, r, r), y);
-    }
-    static __device__ __forceinline__ double sqrt(double a)
-    {
-        const unsigned ex = (unsigned)__double2hiint(a);
-        if (ex - 0x00100000u >= 0x7fe00000u)  // zero and subnormal: a root below 1.5e-154 is dropped; inf, nan
-            return ex < 0x00100000u ? 0.0 : (ex == 0x80000000u ? a : ::sqrt(a));
-        double y;
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-        const double q = __dmul_rn(a, y), r = __fma_rn(-q, y, 1.0);
-        return __fma_rn(__dmul_rn(q, r), __fma_rn(0.375, r, 0.5), q);
-    }
+    // CUDA's correctly rounded reciprocal and root.  (The hardware's
+    // approximations and a third-order step each took 5 % less time, 388
+    // against 409 us a step on 2999 x 701 nodes, with a root up to 0.755 ulp
+    // off.)
+    static __device__ __forceinline__ double rcp(double a) { return 1.0 / a; }
+    static __device__ __forceinline__ double sqrt(double a) { return ::sqrt(a); }
 };
 
 // Paired FP32 arithmetic on sm_100-class GPUs: one instruction applies the
@@ -223,10 +204,9 @@ enum : int { F_WIND = 1, F_FRICTION = 2, F_CORIOLIS = 4 };
 // and with p = g/2 h eta + s - t/2 (= 3 e^2 (a' + s_xx)), d = p + 3 t / 2,
 // r = d - 3 s / 2 the outgoing values are p +- q_x, r +- q_y on the axes and
 // (d +- 3 w +- (q_x +- q_y)) / 4 on the diagonals, stored without the 1/4
-// (the receivers fold it into a multiply-add).  38 operations with friction
-// (root included), 46 and a longer root before; with update64 the tile
-// kernel's step of a 2999 x 701 channel went from 524 to 390 us, 0.93 of
-// what its operations take at the measured 19 cycles a warp instruction.
+// (the receivers fold it into a multiply-add).  33 operations and the root
+// with friction; with update64 the tile kernel's step of a 2999 x 701 channel
+// went from 524 to 409 us.
 template <int FM>
 __device__ __forceinline__ void derive64(const Coef<double>& c, const Raw<double>& r, Src<double>& s)
 {
@@ -277,7 +257,7 @@ __device__ __forceinline__ void derive64(const Coef<double>& c, const Raw<double
 // since D is static): the streamed sums, then
 //     3 e^2 eta' = own + sum + g/2 (D S_eta - eta S_D),
 //     3 e hu'    = x-sum + g/2 (D X_eta - eta X_D) + 3 f_x.
-// 46 operations (56 and a division before).
+// 43 operations and a reciprocal.
 struct Bed64 {
     double s, x, y;
 };
