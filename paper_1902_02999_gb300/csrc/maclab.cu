@@ -1113,7 +1113,9 @@ BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u
 int setup_window(maclab_t s, const Prepared& P, int sms)
 {
     const bool f64 = s->prec == MACLAB_F64;
-    s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0}}, f64, s->fmode, sms);
+    s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0, (int)P.general.size(),
+                                                (int)P.dirs.size()}},
+                              false, f64, s->fmode, sms);
     if (s->wplan.k == 0) return MACLAB_OK;
     // one allocation: lists, instance table, scratch state
     const auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
@@ -2374,11 +2376,15 @@ cudaError_t batch_march(maclab_batch_t b, int par, cudaStream_t st)
 // Strip blocks of a batch for the row march: per instance and strip the rows
 // that hold a node that is not solid, cut into tall blocks and short ones,
 // listed tall first as for a single grid (setup_march).  Left to the tile kernel
-// when a Dirichlet node's inward node falls into another strip block (rows:
-// S or N edge) or the packed arrays pass 2^31 elements.
+// where that is the faster one (window.h: below about a million nodes, and
+// where widths fill tiles but not 60-column strips), when a Dirichlet node's
+// inward node falls into another strip block (rows: S or N edge), or when the
+// packed arrays pass 2^31 elements.
 cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, int sms)
 {
     if (b->total_np >= (size_t)1 << 31) return cudaSuccess;
+    const double tile_us = window::batch_tile_us(b->total_tiles, b->n_general, b->n_dir);
+    if (tile_us <= window::batch_march_us(0, 0, b->n_general, b->n_dir)) return cudaSuccess;
     const size_t smem = march::WARPS * sizeof(march::BatchWarpSmem);
     int nb = 0;
     cudaError_t e = cudaSuccess;
@@ -2452,6 +2458,7 @@ cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, 
     blocks.insert(blocks.end(), low.begin(), low.end());
     std::vector<int> item_of_row(at.back(), -1);
     std::vector<int4> items;
+    double read[2] = {0, 0};  // rows read by plain strip blocks and by the others
     for (size_t t = 0; t < blocks.size(); ++t) {
         const Segment& sg = segs[blocks[t].seg];
         const Prepared& p = P[sg.inst];
@@ -2462,8 +2469,9 @@ cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, 
             plain = plain && !(rowflag[at[blocks[t].seg] + j] & 2);
         }
         items.push_back(make_int4(sg.inst, x0, j0, j1 | (plain ? 1 << 30 : 0)));
+        read[plain ? 0 : 1] += j1 - j0 + 2;
     }
-    if (items.empty()) return cudaSuccess;
+    if (items.empty() || tile_us <= window::batch_march_us(read[0], read[1], b->n_general, b->n_dir)) return cudaSuccess;
     auto item_of = [&](int i, int x, int y) {
         return item_of_row[at[first[i] + (x + shift[i]) / march::OUT] + y];
     };
@@ -2823,13 +2831,14 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         std::vector<window::GridView> views;
         int fmode = 0, dev = 0, sms = 0;
         for (int i = 0; i < count; ++i) {
-            views.push_back(window::GridView{P[i].nx, P[i].ny, P[i].pitch, P[i].bc.edge, P[i].type.data(), (long long)b->off[i]});
+            views.push_back(window::GridView{P[i].nx, P[i].ny, P[i].pitch, P[i].bc.edge, P[i].type.data(), (long long)b->off[i],
+                                             (int)P[i].general.size(), (int)P[i].dirs.size()});
             fmode |= P[i].fmode;
         }
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         b->mfm = fmode;
-        b->wplan = window::make_plan(views, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
+        b->wplan = window::make_plan(views, true, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
         if (b->prec == MACLAB_F32 && b->wplan.k == 0) {
             ce = setup_batch_march(b, P, sms > 0 ? sms : 152);
             if (ce != cudaSuccess) {

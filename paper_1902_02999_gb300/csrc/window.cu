@@ -81,7 +81,7 @@ int cut(int n, int nt, int i) { return (int)((int64_t)n * i / nt); }
 
 }  // namespace
 
-Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
+Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmode, int sms)
 {
     Plan best;
     int64_t nodes = 0;
@@ -201,16 +201,24 @@ Plan make_plan(const std::vector<GridView>& grids, bool f64, int fmode, int sms)
                 }
             }
         }
-    // against one launch per step (us, measured on a GB300): FP32 the row
-    // march, 9.9 us at 512 x 256 nodes, 10.9 at 512 x 512, 13.6 at 1024 x 1024
-    // (a batch's tile kernel 114 for 8 M nodes); FP64 the tile kernel, 29 us
-    // for every full round of the chip's SMs (31 at 512 x 256, 58 at 512 x 512)
-    int64_t tiles64 = 0;
-    for (const GridView& g : grids)
-        tiles64 += (int64_t)((g.nx + tile::TX - 1) / tile::TX) * ((g.ny + tile::TY - 1) / tile::TY);
-    const double single = f64 ? 29.0 * std::max(1.0, std::ceil((double)tiles64 / sms))
-                              : grids.size() > 1 ? 6.0 + nodes / 75e3 : 9.5 + nodes / 220e3;
-    if (best.k == 0 || best_cost / 2070.0 > 0.9 * single) return Plan();
+    // against one launch per step (us, measured on a GB300): an FP32 handle's
+    // row march, 9.9 us at 512 x 256 nodes, 10.9 at 512 x 512, 13.6 at 1024 x
+    // 1024; an FP32 batch's tile kernel (below the node limit above the row
+    // march is the slower one); the FP64 tile kernel, 29 us for every full
+    // round of the chip's SMs (31 at 512 x 256, 58 at 512 x 512).  The model
+    // counts a batch's many waves of blocks up to 1.4 times too dear: of 42
+    // batches up to 640 k nodes this path was the faster one on all where it
+    // came to less than 1.15 of the tile kernel, but for 97 of 64 x 48 (5.5
+    // against 4.4 us).
+    double tiles64 = 0, links = 0, fixed = 0;
+    for (const GridView& g : grids) {
+        tiles64 += (double)((g.nx + tile::TX - 1) / tile::TX) * ((g.ny + tile::TY - 1) / tile::TY);
+        links += g.walls;
+        fixed += g.dirichlet;
+    }
+    const double single = f64 ? 29.0 * std::max(1.0, std::ceil(tiles64 / sms))
+                              : batch ? batch_tile_us(tiles64, links, fixed) : 9.5 + nodes / 220e3;
+    if (best.k == 0 || best_cost / 2070.0 > (batch && !f64 ? 1.15 : 0.9) * single) return Plan();
     best.fm = (fmode & F_CORIOLIS) ? 7 : (fmode & F_FRICTION) ? 3 : 1;
     for (size_t i = 0; i < grids.size(); ++i) {
         const GridView& g = grids[i];
