@@ -185,10 +185,10 @@ int maclab_set_stream(maclab_t sim, void* stream);
 
 /* Advance n >= 0 steps (procedure steps (c)-(e) of Section 3): on small
  * grids several steps per launch (each block steps a tile with a halo of
- * several nodes in shared memory), otherwise one launch of the fused step
- * kernel per step, plus the Dirichlet kernel when the grid has Dirichlet
- * nodes it does not handle itself.  Results are bitwise identical either
- * way.  Asynchronous on the handle's stream. */
+ * several nodes in shared memory; not for calls of fewer steps than make
+ * up for loading the tiles), otherwise one launch of the fused step kernel per
+ * step, plus the Dirichlet kernel when the grid has Dirichlet nodes it does not
+ * handle itself.  Results are bitwise identical either way.  Asynchronous on the handle's stream. */
 int maclab_step(maclab_t sim, int64_t n);
 
 /* Steps per CUDA-graph replay in maclab_step (an even number, 0 = off;

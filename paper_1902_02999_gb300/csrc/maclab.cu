@@ -495,9 +495,10 @@ int launch_pair(maclab_t s)
     return MACLAB_OK;
 }
 
-bool use_window(const maclab_s* s)
+// Whether n steps are taken several per launch.
+bool use_window(const maclab_s* s, int64_t n)
 {
-    return s->wplan.k > 0 && !s->kernel_chosen && s->tblock == 1 && !s->elab && !s->newlevel;
+    return s->wplan.k > 0 && n >= s->wplan.min_steps && !s->kernel_chosen && s->tblock == 1 && !s->elab && !s->newlevel;
 }
 
 // Steps of each of the launches that take n steps at most k at a time: one
@@ -506,7 +507,7 @@ bool use_window(const maclab_s* s)
 // handle's two buffers, where the residual looks for them).
 struct WindowRun {
     int64_t launches, base, more;
-    WindowRun(int64_t n, int k) : launches(std::max<int64_t>(n > 1 ? 2 : 1, (n + k - 1) / k)), base(n / launches), more(n % launches) {}
+    WindowRun(int64_t n, int k) : launches(window::launches(n, k)), base(n / launches), more(n % launches) {}
     int steps(int64_t i) const { return (int)(base + (i < more ? 1 : 0)); }
     bool to_scratch(int64_t i) const { return (launches - 2 - i) % 2 == 0; }  // i < launches - 1
 };
@@ -580,7 +581,7 @@ int advance_window(maclab_t s, int64_t n)
 // n steps: pairs where temporal blocking is on, the last step always single
 int advance(maclab_t s, int64_t n)
 {
-    if (n > 0 && use_window(s))
+    if (n > 0 && use_window(s, n))
         return s->prec == MACLAB_F32 ? advance_window<float>(s, n) : advance_window<double>(s, n);
     const bool pairs_on = s->tblock == 2 && s->prec == MACLAB_F32 && !s->elab && !s->newlevel;
     const int64_t pairs = pairs_on && n >= 3 ? (n - 1) / 2 : 0;
@@ -1526,7 +1527,9 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
     if (rc == MACLAB_OK && s->wplan.k > 0) {
         s->tblock = 1;
         s->kernel_chosen = false;
-        if (use_window(s)) {
+        const int min_steps = s->wplan.min_steps;
+        s->wplan.min_steps = 1;  // however short the trial
+        if (use_window(s, trial_steps)) {
             rc = maclab_step(s, 2);
             cudaEventRecord(e0, s->stream);
             if (rc == MACLAB_OK) rc = maclab_step(s, trial_steps);
@@ -1536,6 +1539,7 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
             cudaEventElapsedTime(&ms, e0, e1);
             keep_window = rc == MACLAB_OK && ms < best;
         }
+        s->wplan.min_steps = min_steps;
     }
     s->kernel_chosen = rc == MACLAB_OK ? !keep_window : chosen0;
     s->events_used = 0;
@@ -2568,7 +2572,7 @@ int batch_window(maclab_batch_t b, int64_t n, cudaStream_t st)
 int batch_steps(maclab_batch_t b, int64_t n, cudaStream_t st)
 {
     const bool f32 = b->prec == MACLAB_F32;
-    if (n > 0 && b->wplan.k > 0) return f32 ? batch_window<float>(b, n, st) : batch_window<double>(b, n, st);
+    if (n > 0 && b->wplan.k > 0 && n >= b->wplan.min_steps) return f32 ? batch_window<float>(b, n, st) : batch_window<double>(b, n, st);
     for (int64_t k = 0; k < n; ++k) {
         const int rc = f32 ? batch_launch<float>(b, st) : batch_launch<double>(b, st);
         if (rc != MACLAB_OK) return rc;

@@ -117,7 +117,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
     static const int TH[] = {2, 4, 8, 12, 16, 24, 32, 48};
     static const int KS[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
     const size_t per_cell = f64 ? cell_bytes<double>() : cell_bytes<float>();
-    double best_cost = 1e300;
+    double best_cost = 1e300, one_step = 0;
     int btw = 0, bth = 0;
     for (int tw : TW)
         for (int th : TH) {
@@ -178,19 +178,25 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
                 const int fit = std::max(1, std::min((int)(MAX_SMEM / smem), 65536 / (128 * threads)));
                 const int64_t per_sm = (wet + sms - 1) / sms;
                 const double waves = (double)((per_sm + fit - 1) / fit), shared = (double)std::min<int64_t>(per_sm, fit);
-                double cyc = LOAD_CELL * ww * wh * shared;
+                double cyc = LOAD_CELL * ww * wh * shared, first = 0;  // first: with the last step alone
                 const double ghosts = (mw >= ww ? 2.0 * wh : 0) + (mh >= wh ? 2.0 * ww : 0);
                 for (int m = k; m >= 1; --m) {
                     // nodes derived and updated with m steps to take
                     const double da = std::min(ww, mw + 2 * m) * (double)std::min(wh, mh + 2 * m);
                     const double db = std::min(ww, mw + 2 * m - 2) * (double)std::min(wh, mh + 2 * m - 2);
-                    cyc += f64 ? f64_cycles(da + ghosts, DERIVE_F64, shared) + f64_cycles(db, UPDATE_F64, shared)
-                               : f32_cycles(0.5 * da, threads, shared) + f32_cycles(0.5 * db, threads, shared);
+                    const double step = f64 ? f64_cycles(da + ghosts, DERIVE_F64, shared) + f64_cycles(db, UPDATE_F64, shared)
+                                            : f32_cycles(0.5 * da, threads, shared) + f32_cycles(0.5 * db, threads, shared);
+                    if (m == 1) first = LOAD_CELL * ww * wh * shared + step;
+                    cyc += step;
                 }
                 // with several blocks on an SM one block's loads hide behind another's steps
-                const double cost = (LAUNCH_CYCLES + (fit > 1 ? BLOCK_CYCLES + waves * cyc : waves * (BLOCK_CYCLES + cyc))) / k;
+                auto whole = [&](double c) {
+                    return LAUNCH_CYCLES + (fit > 1 ? BLOCK_CYCLES + waves * c : waves * (BLOCK_CYCLES + c));
+                };
+                const double cost = whole(cyc) / k;
                 if (cost < best_cost) {
                     best_cost = cost;
+                    one_step = whole(first);
                     best.k = k;
                     best.np = np;
                     best.threads = threads;
@@ -219,6 +225,20 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
     const double single = f64 ? 29.0 * std::max(1.0, std::ceil(tiles64 / sms))
                               : batch ? batch_tile_us(tiles64, links, fixed) : 9.5 + nodes / 220e3;
     if (best.k == 0 || best_cost / 2070.0 > (batch && !f64 ? 1.15 : 0.9) * single) return Plan();
+    // A launch costs its loads and stores however few steps it takes, and a
+    // call of a few steps has no graph replay: two us more for each single-step
+    // launch, and up to five where a handle's row march has wall links (700 x 700
+    // nodes: 12.5 without, 20.1 with walls around).  The fewest steps that this
+    // path takes in less (0.9: the model counts a one-step launch a tenth too
+    // dear or more).  One step: 809 x 809 nodes 16.3 us here, 13.0 on the row
+    // march; four 256 x 256 grids 8.8, tiles 6.7; 600 x 600 12.4 both; 700 x 700
+    // with walls 15.5 here.
+    const double alone = single + 2.0 + (!f64 && !batch && links > 0 ? 0.5 + std::min(4.5, links / 500) : 0.0);
+    const double more = best.k > 1 ? (best_cost * best.k - one_step) / (best.k - 1) : one_step;
+    for (; best.min_steps < 64; ++best.min_steps) {
+        const int64_t n = best.min_steps, l = launches(n, best.k);
+        if (0.9 * (l * one_step + (n - l) * more) / 2070.0 <= n * alone) break;
+    }
     best.fm = (fmode & F_CORIOLIS) ? 7 : (fmode & F_FRICTION) ? 3 : 1;
     for (size_t i = 0; i < grids.size(); ++i) {
         const GridView& g = grids[i];

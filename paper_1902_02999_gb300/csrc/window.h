@@ -4,6 +4,8 @@
 #pragma once
 #include "maclab_window.cuh"
 
+#include <algorithm>
+#include <cstdint>
 #include <vector>
 
 namespace maclab {
@@ -41,9 +43,14 @@ struct Plan {
     int np = 1, threads = 0;  // kernel variant (FP32 pairs per thread) and block size
     int fm = 0;               // force terms compiled in
     size_t smem = 0;
+    int min_steps = 1;        // shorter calls are cheaper in single-step launches
     Shape shape{};
     std::vector<Item> items;
 };
+
+// Launches that take n steps at most k at a time: one for a single step, two
+// or more otherwise (see WindowRun).
+inline int64_t launches(int64_t n, int k) { return std::max<int64_t>(n > 1 ? 2 : 1, (n + k - 1) / k); }
 
 // Tiles and steps per launch for these grids, a batch's or one handle's
 // (plan.k = 0 when the single-step kernels are the better choice).
