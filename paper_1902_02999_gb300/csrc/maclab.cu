@@ -1118,12 +1118,16 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
                                                 (int)P.dirs.size()}},
                               false, f64, s->fmode, sms);
     if (s->wplan.k == 0) return MACLAB_OK;
-    // one allocation: lists, instance table, scratch state
+    // one allocation: lists, instance table, scratch state; without it every
+    // step is a launch of its own
     const auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
     const size_t NP = (size_t)P.pitch * P.ny, state = up(NP * s->esize), lists = up(window::list_bytes(s->wplan));
     const size_t inst = up(f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>));
     unsigned char* mem = (unsigned char*)dev_alloc(s, lists + inst + 3 * state);
-    if (!mem) return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
+    if (!mem) {
+        s->wplan = window::Plan();
+        return MACLAB_OK;
+    }
     s->winst = mem + lists;
     for (int q = 0; q < 3; ++q) s->wmid[q] = mem + lists + inst + q * state;
     cudaError_t e = cudaSuccess;
@@ -2501,18 +2505,23 @@ cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, 
         gn.insert(gn.end(), p.general.begin(), p.general.end());
     }
     march::BatchGeom g{};
-    auto put = [&](const void* src, size_t bytes) -> void* {
-        void* p = bdev_alloc(b, bytes);
-        if (!p) e = cudaErrorMemoryAllocation;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, b->stream);
-        return p;
-    };
-    g.items = (const int4*)put(items.data(), items.size() * sizeof(int4));
-    if (!gn.empty()) g.glist = (const int*)put(gn.data(), gn.size() * sizeof(int));
-    if (any_d) {
-        g.dstart = (const int*)put(ds.data(), ds.size() * sizeof(int));
-        g.dlist = (const DirNode*)put(dn.data(), dn.size() * sizeof(DirNode));
+    const auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
+    const size_t sizes[4] = {items.size() * sizeof(int4), gn.size() * sizeof(int), any_d ? ds.size() * sizeof(int) : 0,
+                             dn.size() * sizeof(DirNode)};
+    const void* from[4] = {items.data(), gn.data(), ds.data(), dn.data()};
+    void* at_dev[4] = {};
+    unsigned char* mem = (unsigned char*)bdev_alloc(b, up(sizes[0]) + up(sizes[1]) + up(sizes[2]) + up(sizes[3]));
+    if (!mem) return cudaSuccess;  // the tiles need no lists
+    for (int k = 0; k < 4; ++k) {
+        if (sizes[k] == 0) continue;
+        at_dev[k] = mem;
+        mem += up(sizes[k]);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(at_dev[k], from[k], sizes[k], cudaMemcpyHostToDevice, b->stream);
     }
+    g.items = (const int4*)at_dev[0];
+    g.glist = (const int*)at_dev[1];
+    g.dstart = (const int*)at_dev[2];
+    g.dlist = (const DirNode*)at_dev[3];
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return e;
     g.nitems = (int)items.size();
@@ -2841,36 +2850,29 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         }
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int n_sms = sms > 0 ? sms : 152;
         b->mfm = fmode;
-        b->wplan = window::make_plan(views, true, b->prec == MACLAB_F64, fmode, sms > 0 ? sms : 152);
-        if (b->prec == MACLAB_F32 && b->wplan.k == 0) {
-            ce = setup_batch_march(b, P, sms > 0 ? sms : 152);
-            if (ce != cudaSuccess) {
-                const int code = ce == cudaErrorMemoryAllocation ? MACLAB_E_NOMEM : MACLAB_E_CUDA;
-                bfail(nullptr, code, std::string("batch row march: ") + cudaGetErrorString(ce));
-                brelease(b);
-                delete b;
-                return code;
+        b->wplan = window::make_plan(views, true, b->prec == MACLAB_F64, fmode, n_sms);
+        // the several-step path and the row march need memory of their own; where
+        // it cannot be had the batch takes the next path
+        if (b->wplan.k > 0) {
+            const size_t lists = window::list_bytes(b->wplan), state = (NP * b->esize + 255) & ~size_t(255);
+            unsigned char* mem = (unsigned char*)bdev_alloc(b, lists + 3 * state);
+            if (mem) {
+                for (int q = 0; q < 3; ++q) b->wmid[q] = mem + lists + q * state;
+                ce = b->prec == MACLAB_F32 ? window::build_lists<float>(b->wplan, b->insts, mem, b->stream, &b->wlists)
+                                           : window::build_lists<double>(b->wplan, b->insts, mem, b->stream, &b->wlists);
+                if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
+            } else {
+                b->wplan = window::Plan();
             }
         }
-        if (b->wplan.k > 0) {
-            void* mem = bdev_alloc(b, window::list_bytes(b->wplan));
-            bool got = mem != nullptr;
-            for (int q = 0; q < 3 && got; ++q) got = (b->wmid[q] = bdev_alloc(b, NP * b->esize)) != nullptr;
-            if (!got) {
-                brelease(b);
-                delete b;
-                return bfail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
-            }
-            ce = b->prec == MACLAB_F32 ? window::build_lists<float>(b->wplan, b->insts, mem, b->stream, &b->wlists)
-                                       : window::build_lists<double>(b->wplan, b->insts, mem, b->stream, &b->wlists);
-            if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
-            if (ce != cudaSuccess) {
-                bfail(nullptr, MACLAB_E_CUDA, std::string("batch upload: ") + cudaGetErrorString(ce));
-                brelease(b);
-                delete b;
-                return MACLAB_E_CUDA;
-            }
+        if (ce == cudaSuccess && b->prec == MACLAB_F32 && b->wplan.k == 0) ce = setup_batch_march(b, P, n_sms);
+        if (ce != cudaSuccess) {
+            bfail(nullptr, MACLAB_E_CUDA, std::string("batch upload: ") + cudaGetErrorString(ce));
+            brelease(b);
+            delete b;
+            return MACLAB_E_CUDA;
         }
     }
     *out = b;
