@@ -57,9 +57,9 @@ struct maclab_s {
     void* eta[2] = {nullptr, nullptr};
     void* u[2] = {nullptr, nullptr};
     void* v[2] = {nullptr, nullptr};
-    void* D = nullptr;         // still-water depth in the state precision
+    void* D = nullptr;         // still-water depth in the state precision (FP64: D64)
     double* D64 = nullptr;     // still-water depth in double
-    double* bed = nullptr;     // FP64: stencils of D, three planes
+    double* bed = nullptr;     // FP64: stencils of D, three planes (nullptr: no memory for them)
     uint8_t* type = nullptr;
     int* general = nullptr;    // node indices (j * nx + i) of general-link nodes
     int n_general = 0;
@@ -117,6 +117,7 @@ struct maclab_s {
     bool kernel_chosen = false;    // the caller picked a step kernel: every step is a launch of it
     window::Plan wplan;            // k = 0: not used on this grid
     window::Lists wlists{};
+    void* wmem = nullptr;          // the path's memory: lists, then
     void* winst = nullptr;         // BatchInst<T>[1]
     void* wmid[3] = {nullptr, nullptr, nullptr};  // state between launches
     std::vector<cudaEvent_t> events;  // pairs around step-kernel launches
@@ -160,6 +161,31 @@ void* dev_alloc(maclab_t s, size_t bytes)
         s->device_bytes += bytes;
     }
     return p;
+}
+
+void dev_free(maclab_t s, void* p)
+{
+    for (size_t q = 0; q < s->bufs.size(); ++q) {
+        if (s->bufs[q].p != p) continue;
+        if (s->has_alloc)
+            s->alloc.release(p, s->alloc.ctx);
+        else
+            cudaFree(p);
+        s->device_bytes -= s->bufs[q].bytes;
+        s->bufs.erase(s->bufs.begin() + q);
+        return;
+    }
+}
+
+// Memory for what only makes steps faster: kept where a marked state's copy
+// still fits beside it.
+void* dev_alloc_extra(maclab_t s, size_t bytes)
+{
+    void* p = dev_alloc(s, bytes);
+    if (!p) return nullptr;
+    void* mark = dev_alloc(s, 3 * (size_t)s->pitch * s->grid.ny * s->esize);
+    dev_free(s, mark ? mark : p);
+    return mark ? p : nullptr;
 }
 
 void release_all(maclab_t s)
@@ -1114,6 +1140,7 @@ BatchInst<T> make_inst(const Prepared& P, void* const (&eta)[2], void* const (&u
 int setup_window(maclab_t s, const Prepared& P, int sms)
 {
     const bool f64 = s->prec == MACLAB_F64;
+    if (f64 && !s->bed) return MACLAB_OK;  // (the path's FP64 form reads the stencils)
     s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0, (int)P.general.size(),
                                                 (int)P.dirs.size()}},
                               false, f64, s->fmode, sms);
@@ -1123,11 +1150,12 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     const auto up = [](size_t n) { return (n + 255) & ~size_t(255); };
     const size_t NP = (size_t)P.pitch * P.ny, state = up(NP * s->esize), lists = up(window::list_bytes(s->wplan));
     const size_t inst = up(f64 ? sizeof(BatchInst<double>) : sizeof(BatchInst<float>));
-    unsigned char* mem = (unsigned char*)dev_alloc(s, lists + inst + 3 * state);
+    unsigned char* mem = (unsigned char*)dev_alloc_extra(s, lists + inst + 3 * state);
     if (!mem) {
         s->wplan = window::Plan();
         return MACLAB_OK;
     }
+    s->wmem = mem;
     s->winst = mem + lists;
     for (int q = 0; q < 3; ++q) s->wmid[q] = mem + lists + inst + q * state;
     cudaError_t e = cudaSuccess;
@@ -1222,11 +1250,11 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
         ok = (s->eta[k] = dev_alloc(s, NP * s->esize)) && (s->u[k] = dev_alloc(s, NP * s->esize)) &&
              (s->v[k] = dev_alloc(s, NP * s->esize));
     }
-    ok = ok && (s->D = dev_alloc(s, NP * s->esize)) && (s->D64 = (double*)dev_alloc(s, NP * 8)) &&
+    ok = ok && (s->D64 = (double*)dev_alloc(s, NP * 8)) &&
+         (s->D = s->prec == MACLAB_F64 ? s->D64 : dev_alloc(s, NP * s->esize)) &&
          (s->type = (uint8_t*)dev_alloc(s, NP + 64)) && (s->stage = (double*)dev_alloc(s, 3 * N * 8)) &&
          (s->partial = (double*)dev_alloc(s, (size_t)s->red_blocks * RED_NVAL * 8)) &&
          (s->red_out = (double*)dev_alloc(s, RED_NVAL * 8));
-    if (ok && s->prec == MACLAB_F64) ok = (s->bed = (double*)dev_alloc(s, 3 * NP * 8)) != nullptr;
     if (ok && s->prec == MACLAB_F32) ok = (s->tma_err = (int*)dev_alloc(s, sizeof(int))) != nullptr;
     if (ok && !general.empty())
         ok = (s->general = (int*)dev_alloc(s, general.size() * sizeof(int))) &&
@@ -1239,6 +1267,7 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
         delete s;
         return fail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
     }
+    if (s->prec == MACLAB_F64) s->bed = (double*)dev_alloc_extra(s, 3 * NP * 8);
     s->n_general = (int)general.size();
     s->n_dir = (int)dirs.size();
 
@@ -1254,8 +1283,6 @@ int maclab_create(const maclab_grid* grid, const maclab_params* params, const ma
         for (size_t k = 0; k < NP; ++k) Df[k] = (float)D64[k];
         put(s->D, Df.data(), NP * 4);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s->stream);
-    } else {
-        put(s->D, D64.data(), NP * 8);
     }
     std::vector<uint8_t> tpad(type);
     tpad.resize(NP + 64, 0);
@@ -1561,17 +1588,7 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
     drop_graphs(s);
     for (int k = 0; k < 6; ++k) cudaMemcpyAsync(src[k], keep[k], bytes, cudaMemcpyDeviceToDevice, s->stream);
     cudaStreamSynchronize(s->stream);
-    for (int k = 0; k < 6; ++k) {  // give the scratch back
-        for (size_t q = 0; q < s->bufs.size(); ++q) {
-            if (s->bufs[q].p == keep[k]) {
-                if (s->has_alloc) s->alloc.release(keep[k], s->alloc.ctx);
-                else cudaFree(keep[k]);
-                s->device_bytes -= s->bufs[q].bytes;
-                s->bufs.erase(s->bufs.begin() + q);
-                break;
-            }
-        }
-    }
+    for (int k = 0; k < 6; ++k) dev_free(s, keep[k]);
     s->cur = cur;
     s->n = n0;
     s->have_prev = hp;
@@ -1893,9 +1910,22 @@ int maclab_set_relaxation(maclab_t s, double tau)
             if (kind != K_SOLID && kind != K_FLUID)
                 return fail(s, MACLAB_E_ARG, "the distribution form takes fluid and solid nodes only");
         }
-    for (int k = 0; k < 2; ++k)
-        if (!s->gdist[k] && !(s->gdist[k] = dev_alloc(s, 9 * NP * s->esize)))
-            return fail(s, MACLAB_E_NOMEM, "distribution buffers");
+    for (int k = 0; k < 2; ++k) {
+        if (!s->gdist[k]) s->gdist[k] = dev_alloc(s, 9 * NP * s->esize);
+        if (!s->gdist[k] && (s->bed || s->wmem)) {
+            // what makes the other form's steps faster makes room
+            e = cudaStreamSynchronize(s->stream);
+            if (e != cudaSuccess) return cuda_fail(s, e, "relaxation setup");
+            drop_graphs(s);
+            dev_free(s, s->bed);
+            dev_free(s, s->wmem);
+            s->bed = nullptr;
+            s->wmem = nullptr;
+            s->wplan = window::Plan();
+            s->gdist[k] = dev_alloc(s, 9 * NP * s->esize);
+        }
+        if (!s->gdist[k]) return fail(s, MACLAB_E_NOMEM, "distribution buffers");
+    }
     cudaError_t ae = cudaSuccess;
     const size_t smem = s->prec == MACLAB_F32 ? sizeof(elab::Smem<float>) : sizeof(elab::Smem<double>);
 #define MACLAB_ATTR(m)                                                                                        \
@@ -2184,9 +2214,9 @@ struct maclab_batch_s {
     void* eta[2] = {nullptr, nullptr};
     void* u[2] = {nullptr, nullptr};
     void* v[2] = {nullptr, nullptr};
-    void* D = nullptr;
+    void* D = nullptr;              // (FP64: D64)
     double* D64 = nullptr;
-    double* bed = nullptr;          // FP64: stencils of D, three packed planes
+    double* bed = nullptr;          // FP64: stencils of D, three packed planes (nullptr: no memory for them)
     uint8_t* type = nullptr;
     double* stage = nullptr;
     void* insts = nullptr;          // BatchInst<T>[count]
@@ -2253,6 +2283,29 @@ void* bdev_alloc(maclab_batch_t b, size_t bytes)
         b->device_bytes += bytes;
     }
     return p;
+}
+
+void bdev_free(maclab_batch_t b, void* p)
+{
+    for (size_t q = 0; q < b->bufs.size(); ++q) {
+        if (b->bufs[q].p != p) continue;
+        if (b->has_alloc)
+            b->alloc.release(p, b->alloc.ctx);
+        else
+            cudaFree(p);
+        b->device_bytes -= b->bufs[q].bytes;
+        b->bufs.erase(b->bufs.begin() + q);
+        return;
+    }
+}
+
+void* bdev_alloc_extra(maclab_batch_t b, size_t bytes)  // as dev_alloc_extra
+{
+    void* p = bdev_alloc(b, bytes);
+    if (!p) return nullptr;
+    void* mark = bdev_alloc(b, 3 * b->total_np * b->esize);
+    bdev_free(b, mark ? mark : p);
+    return mark ? p : nullptr;
 }
 
 void brelease(maclab_batch_t b)
@@ -2510,7 +2563,7 @@ cudaError_t setup_batch_march(maclab_batch_t b, const std::vector<Prepared>& P, 
                              dn.size() * sizeof(DirNode)};
     const void* from[4] = {items.data(), gn.data(), ds.data(), dn.data()};
     void* at_dev[4] = {};
-    unsigned char* mem = (unsigned char*)bdev_alloc(b, up(sizes[0]) + up(sizes[1]) + up(sizes[2]) + up(sizes[3]));
+    unsigned char* mem = (unsigned char*)bdev_alloc_extra(b, up(sizes[0]) + up(sizes[1]) + up(sizes[2]) + up(sizes[3]));
     if (!mem) return cudaSuccess;  // the tiles need no lists
     for (int k = 0; k < 4; ++k) {
         if (sizes[k] == 0) continue;
@@ -2749,7 +2802,8 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         ok = (b->eta[k] = bdev_alloc(b, NP * b->esize)) && (b->u[k] = bdev_alloc(b, NP * b->esize)) &&
              (b->v[k] = bdev_alloc(b, NP * b->esize));
     const size_t inst_bytes = b->prec == MACLAB_F32 ? sizeof(BatchInst<float>) : sizeof(BatchInst<double>);
-    ok = ok && (b->D = bdev_alloc(b, NP * b->esize)) && (b->D64 = (double*)bdev_alloc(b, NP * 8)) &&
+    ok = ok && (b->D64 = (double*)bdev_alloc(b, NP * 8)) &&
+         (b->D = b->prec == MACLAB_F64 ? b->D64 : bdev_alloc(b, NP * b->esize)) &&
          (b->type = (uint8_t*)bdev_alloc(b, NP + 64)) && (b->stage = (double*)bdev_alloc(b, 3 * maxN * 8)) &&
          (b->insts = bdev_alloc(b, inst_bytes * count)) &&
          (b->tile_inst = (int*)bdev_alloc(b, tile_inst.size() * sizeof(int))) &&
@@ -2758,7 +2812,6 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
          (b->red_out = (double*)bdev_alloc(b, (size_t)count * RED_NVAL * 8)) &&
          (b->barrier = (GridBarrier*)bdev_alloc(b, sizeof(GridBarrier))) &&
          (b->persist_err = (int*)bdev_alloc(b, sizeof(int)));
-    if (ok && b->prec == MACLAB_F64) ok = (b->bed = (double*)bdev_alloc(b, 3 * NP * 8)) != nullptr;
     if (ok && b->n_general)
         ok = (b->general = (int2*)bdev_alloc(b, general.size() * sizeof(int2))) &&
              (b->gen_nodes = (int*)bdev_alloc(b, gen_nodes.size() * sizeof(int))) &&
@@ -2772,6 +2825,7 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         delete b;
         return bfail(nullptr, MACLAB_E_NOMEM, "device allocation failed");
     }
+    if (b->prec == MACLAB_F64) b->bed = (double*)bdev_alloc_extra(b, 3 * NP * 8);
     // static data
     std::vector<double> D64(NP, 0.0);
     std::vector<uint8_t> type(NP + 64, 0);
@@ -2789,8 +2843,6 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         Df.resize(NP);
         for (size_t k = 0; k < NP; ++k) Df[k] = (float)D64[k];
         put(b->D, Df.data(), NP * 4);
-    } else {
-        put(b->D, D64.data(), NP * 8);
     }
     put(b->type, type.data(), NP + 64);
     put(b->tile_inst, tile_inst.data(), tile_inst.size() * sizeof(int));
@@ -2814,7 +2866,7 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
     } else {
         fill_insts<double>(b, P, instd);
         put(b->insts, instd.data(), instd.size() * sizeof(BatchInst<double>));
-        for (int i = 0; i < count && ce == cudaSuccess; ++i) {
+        for (int i = 0; i < count && b->bed && ce == cudaSuccess; ++i) {
             bed_stencil_kernel<<<grid_blocks((size_t)b->nodes[i], 256, 4096), 256, 0, b->stream>>>(
                 instd[i].f[0], b->bed + b->off[i], NP);
             ce = cudaGetLastError();
@@ -2852,12 +2904,12 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int n_sms = sms > 0 ? sms : 152;
         b->mfm = fmode;
-        b->wplan = window::make_plan(views, true, b->prec == MACLAB_F64, fmode, n_sms);
+        if (b->prec == MACLAB_F32 || b->bed) b->wplan = window::make_plan(views, true, b->prec == MACLAB_F64, fmode, n_sms);
         // the several-step path and the row march need memory of their own; where
         // it cannot be had the batch takes the next path
         if (b->wplan.k > 0) {
             const size_t lists = window::list_bytes(b->wplan), state = (NP * b->esize + 255) & ~size_t(255);
-            unsigned char* mem = (unsigned char*)bdev_alloc(b, lists + 3 * state);
+            unsigned char* mem = (unsigned char*)bdev_alloc_extra(b, lists + 3 * state);
             if (mem) {
                 for (int q = 0; q < 3; ++q) b->wmid[q] = mem + lists + q * state;
                 ce = b->prec == MACLAB_F32 ? window::build_lists<float>(b->wplan, b->insts, mem, b->stream, &b->wlists)

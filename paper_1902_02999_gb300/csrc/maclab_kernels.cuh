@@ -287,9 +287,22 @@ __device__ __forceinline__ void update64(const Coef<double>& K, double cL1, doub
     ou = noslip ? 0.0 : O::mul(mx, inv);
     ov = noslip ? 0.0 : O::mul(my, inv);
 }
-__device__ __forceinline__ Bed64 bed_at(const Fields<double>& f, size_t i)
+// The stencils from the depths of the eight sources, d_a = D(x - c_a).
+__device__ __forceinline__ Bed64 bed_of(double d1, double d2, double d3, double d4, double d5, double d6, double d7,
+                                        double d8)
 {
-    return Bed64{f.bed[i], f.bed[i + f.bed_plane], f.bed[i + 2 * f.bed_plane]};
+    using O = Op<double>;
+    const double L = O::fma(0.25, O::add(d2, d8), d1), R = O::fma(0.25, O::add(d4, d6), d5);
+    return Bed64{O::add(O::add(L, R), O::add(d3, d7)), O::sub(L, R),
+                 O::fma(0.25, O::sub(O::add(d2, d4), O::add(d8, d6)), O::sub(d3, d7))};
+}
+// Node i's stencils: the planes laid out once per grid, or, where there was no
+// memory for those (f.bed null), from the depths at hand (12 more operations).
+__device__ __forceinline__ Bed64 bed_at(const Fields<double>& f, size_t i, double d1, double d2, double d3, double d4,
+                                        double d5, double d6, double d7, double d8)
+{
+    if (f.bed) return Bed64{f.bed[i], f.bed[i + f.bed_plane], f.bed[i + 2 * f.bed_plane]};
+    return bed_of(d1, d2, d3, d4, d5, d6, d7, d8);
 }
 
 // Source-side quantities of one node (see the header comment).
@@ -747,7 +760,7 @@ __device__ __forceinline__ void emit_row(const Fields<T>& f, int j, int xl, int 
             const size_t at = ok && j < f.ny ? (size_t)j * f.pitch + x : 0;
             update64(K, cL.o1, mL.o2, pL.o8, cR.o5, mR.o4, pR.o6, mC.o3, pC.o7,
                      Eta8{mL.eta, mC.eta, mR.eta, cL.eta, cR.eta, pL.eta, pC.eta, pR.eta}, cC.eta, cC.D, cC.ownh, cC.hFx,
-                     cC.hFy, bed_at(f, at), noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
+                     cC.hFy, bed_at(f, at, cL.D, mL.D, mC.D, mR.D, cR.D, pR.D, pC.D, pL.D), noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
         } else {
             using V2 = typename Vec2<T>::type;
             auto ed = [](const Src<T>& q) { return V2{q.eta, q.D}; };
@@ -955,7 +968,7 @@ __device__ __forceinline__ void general_node64(const Fields<double>& f, int i, i
     Src<double> X;
     derive64<ALL>(f.c, Raw<double>{f.eta[xi], f.u[xi], f.v[xi], f.D[xi], 0}, X);
     const double back[9] = {0.0, X.o5, X.o6, X.o7, X.o8, X.o1, X.o2, X.o3, X.o4};
-    double o[9], eta[9];
+    double o[9], eta[9], d[9];
 #pragma unroll
     for (int a = 1; a < 9; ++a) {
         const int cx = (a == 1 || a == 2 || a == 8) - (a == 4 || a == 5 || a == 6);
@@ -965,6 +978,7 @@ __device__ __forceinline__ void general_node64(const Fields<double>& f, int i, i
         const int sj = resolve_index(j - cy, f.ny, f.edge[2], f.edge[3], 2, flip);
         o[a] = back[a];
         eta[a] = X.eta;
+        d[a] = X.D;
         if (si < 0 || sj < 0) continue;
         const size_t s = (size_t)sj * f.pitch + si;
         if ((f.type[s] & KIND_MASK) == K_SOLID) continue;
@@ -972,10 +986,12 @@ __device__ __forceinline__ void general_node64(const Fields<double>& f, int i, i
         derive64<ALL>(f.c, Raw<double>{f.eta[s], f.u[s], f.v[s], f.D[s], flip}, Y);
         o[a] = a == 1 ? Y.o1 : a == 2 ? Y.o2 : a == 3 ? Y.o3 : a == 4 ? Y.o4 : a == 5 ? Y.o5 : a == 6 ? Y.o6 : a == 7 ? Y.o7 : Y.o8;
         eta[a] = Y.eta;
+        d[a] = Y.D;
     }
     update64(f.c, o[1], o[2], o[8], o[5], o[4], o[6], o[3], o[7],
              Eta8{eta[2], eta[3], eta[4], eta[1], eta[5], eta[8], eta[7], eta[6]}, X.eta, X.D, X.ownh, X.hFx, X.hFy,
-             bed_at(f, xi), (f.type[xi] & KIND_MASK) == K_NOSLIP, f.eta1[xi], f.u1[xi], f.v1[xi]);
+             bed_at(f, xi, d[1], d[2], d[3], d[4], d[5], d[6], d[7], d[8]), (f.type[xi] & KIND_MASK) == K_NOSLIP,
+             f.eta1[xi], f.u1[xi], f.v1[xi]);
 }
 
 // U: links taken at a time (their loads are in flight together).
@@ -1057,7 +1073,6 @@ __global__ void __launch_bounds__(128) step_general_kernel(const Fields<T> f, co
 static __global__ void bed_stencil_kernel(const __grid_constant__ Fields<double> f, double* __restrict__ bed,
                                           size_t plane)
 {
-    using O = Op<double>;
     const size_t total = (size_t)f.nx * f.ny;
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < total; k += (size_t)gridDim.x * blockDim.x) {
         const int j = (int)(k / f.nx), i = (int)(k - (size_t)j * f.nx);
@@ -1072,10 +1087,10 @@ static __global__ void bed_stencil_kernel(const __grid_constant__ Fields<double>
             const size_t s = (size_t)sj * f.pitch + si;
             if ((f.type[s] & KIND_MASK) != K_SOLID) d[a] = f.D[s];
         }
-        const double L = O::fma(0.25, O::add(d[2], d[8]), d[1]), R = O::fma(0.25, O::add(d[4], d[6]), d[5]);
-        bed[x] = O::add(O::add(L, R), O::add(d[3], d[7]));
-        bed[x + plane] = O::sub(L, R);
-        bed[x + 2 * plane] = O::fma(0.25, O::sub(O::add(d[2], d[4]), O::add(d[8], d[6])), O::sub(d[3], d[7]));
+        const Bed64 b = bed_of(d[1], d[2], d[3], d[4], d[5], d[6], d[7], d[8]);
+        bed[x] = b.s;
+        bed[x + plane] = b.x;
+        bed[x + 2 * plane] = b.y;
     }
 }
 
@@ -1402,7 +1417,10 @@ __device__ __forceinline__ void tile_phase_bc(const Fields<T>& f, int x0, int y0
             okmask |= (ok ? 1u : 0u) << k;
             const Src<T>& me = own[r][k];
             Bed64 bd{};
-            if constexpr (std::is_same<T, double>::value) bd = bed_at(f, ok ? (size_t)y * f.pitch + x : 0);
+            if constexpr (std::is_same<T, double>::value)
+                bd = bed_at(f, ok ? (size_t)y * f.pitch + x : 0, sm.ed(lr, lc - 1).y, sm.ed(lr - 1, lc - 1).y,
+                            sm.ed(lr - 1, lc).y, sm.ed(lr - 1, lc + 1).y, sm.ed(lr, lc + 1).y, sm.ed(lr + 1, lc + 1).y,
+                            sm.ed(lr + 1, lc).y, sm.ed(lr + 1, lc - 1).y);
             node_update<T>(sm, lr, lc, K, me.eta, me.D, me.ownh, me.hFx, me.hFy,
                            (ty & KIND_MASK) == K_NOSLIP, bd, oe[k], ou[k], ov[k]);
         }

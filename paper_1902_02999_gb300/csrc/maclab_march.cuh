@@ -414,10 +414,14 @@ __device__ __forceinline__ void march_row(const Fields<T>& f, int r, int x, cons
             const size_t at = EDGE ? (size_t)(r - 1) * f.pitch + x : (size_t)(unsigned)((r - 1) * f.pitch + x);
             update64(f.c, A1.x, M2.x, Lo8, C5.x, M4.x, d.o6.y, M3.x, d.o7.x,
                      Eta8{m[0].x, m[1].x, m[2].x, c[0].x, c[2].x, pe[0].x, pe[1].x, pe[2].x}, c[1].x, c[1].y, own.ownh.x,
-                     own.hFx.x, own.hFy.x, bed_at(f, ok & 1u ? at : 0), ns0, oe.x, ou.x, ov.x);
+                     own.hFx.x, own.hFy.x,
+                     bed_at(f, ok & 1u ? at : 0, c[0].y, m[0].y, m[1].y, m[2].y, c[2].y, pe[2].y, pe[1].y, pe[0].y), ns0, oe.x,
+                     ou.x, ov.x);
             update64(f.c, A1.y, M2.y, d.o8.x, C5.y, M4.y, Ro6, M3.y, d.o7.y,
                      Eta8{m[1].x, m[2].x, m[3].x, c[1].x, c[3].x, pe[1].x, pe[2].x, pe[3].x}, c[2].x, c[2].y, own.ownh.y,
-                     own.hFx.y, own.hFy.y, bed_at(f, ok & 2u ? at + 1 : 0), ns1, oe.y, ou.y, ov.y);
+                     own.hFx.y, own.hFy.y,
+                     bed_at(f, ok & 2u ? at + 1 : 0, c[1].y, m[1].y, m[2].y, m[3].y, c[3].y, pe[3].y, pe[2].y, pe[1].y), ns1, oe.y,
+                     ou.y, ov.y);
         }
         const size_t idx = EDGE ? (size_t)(r - 1) * f.pitch + x + (B ? f.boff : 0u)
                                 : (size_t)(unsigned)((r - 1) * f.pitch + x + (B ? f.boff : 0u));
