@@ -1142,7 +1142,7 @@ int setup_window(maclab_t s, const Prepared& P, int sms)
     const bool f64 = s->prec == MACLAB_F64;
     if (f64 && !s->bed) return MACLAB_OK;  // (the path's FP64 form reads the stencils)
     s->wplan = window::make_plan({window::GridView{P.nx, P.ny, P.pitch, P.bc.edge, P.type.data(), 0, (int)P.general.size(),
-                                                (int)P.dirs.size()}},
+                                                (int)P.dirs.size(), P.general.data()}},
                               false, f64, s->fmode, sms);
     if (s->wplan.k == 0) return MACLAB_OK;
     // one allocation: lists, instance table, scratch state; without it every
@@ -2897,7 +2897,7 @@ int maclab_batch_create(int count, const maclab_grid* grids, const maclab_params
         int fmode = 0, dev = 0, sms = 0;
         for (int i = 0; i < count; ++i) {
             views.push_back(window::GridView{P[i].nx, P[i].ny, P[i].pitch, P[i].bc.edge, P[i].type.data(), (long long)b->off[i],
-                                             (int)P[i].general.size(), (int)P[i].dirs.size()});
+                                             (int)P[i].general.size(), (int)P[i].dirs.size(), P[i].general.data()});
             fmode |= P[i].fmode;
         }
         cudaGetDevice(&dev);

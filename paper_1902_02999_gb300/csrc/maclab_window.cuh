@@ -69,7 +69,7 @@ struct Shape {  // shared by every block of a launch (the largest window)
     int rows;    // padded rows
     int units;   // room in a tile's list of units
     int ghosts;  // ... of ghosts
-    int walls;   // ... of nodes with a bounce-back link (FP32)
+    int walls;   // ... of nodes with a bounce-back link (FP32; the most of any tile)
     int dirs;    // ... of Dirichlet nodes
     __host__ __device__ int cells() const { return rows * 2 * hw; }
 };

@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
 
 namespace maclab {
 namespace window {
@@ -39,23 +40,18 @@ double f64_cycles(double nodes, double instructions, double shared)
 }
 
 // nodes that are not solid in [0, x) x [0, y), row length nx + 1 (empty when
-// no node is solid), and whether a node has a bounce-back link
+// no node is solid)
 struct Counts {
     std::vector<int> c;
     int w;
-    bool walls = false;
     explicit Counts(const GridView& g) : w(g.nx + 1)
     {
         bool dry = false;
-        for (int y = 0; y < g.ny; ++y) {
+        for (int y = 0; y < g.ny && !dry; ++y) {
             const uint8_t* t = g.type + (size_t)y * g.pitch;
-            uint8_t any = 0, solid = 0;
-            for (int x = 0; x < g.nx; ++x) {
-                any |= t[x];
-                solid |= (t[x] & KIND_MASK) == K_SOLID;
-            }
-            walls = walls || (any & GENERAL_BIT);
-            dry = dry || solid;
+            uint8_t solid = 0;
+            for (int x = 0; x < g.nx; ++x) solid |= (t[x] & KIND_MASK) == K_SOLID;
+            dry = solid;
         }
         if (!dry) return;
         c.assign((size_t)(g.nx + 1) * (g.ny + 1), 0);
@@ -79,13 +75,38 @@ struct Counts {
 int tiles(int n, int t) { return std::max(1, std::min((n + t - 1) / t, std::max(1, n / 2))); }
 int cut(int n, int nt, int i) { return (int)((int64_t)n * i / nt); }
 
+// The most nodes with a bounce-back link in the window of any of a grid's nt
+// tiles (nodes that windows wrap onto more than once count each time).
+int most_walls(const GridView& g, int ntx, int nty, int k)
+{
+    // per column and row: the tiles whose windows hold it, and how often
+    auto holders = [](int n, int nt, int lo_kind, int hi_kind, int halo) {
+        std::vector<std::vector<std::pair<int, int>>> at(n);
+        for (int t = 0; t < nt; ++t) {
+            const Axis a = make_axis(cut(n, nt, t), cut(n, nt, t + 1), n, lo_kind, hi_kind, halo, 1);
+            for (int i = 0; i < a.n; ++i) {
+                auto& q = at[wrapped(a.lo + i, n)];
+                if (!q.empty() && q.back().first == t) ++q.back().second;
+                else q.emplace_back(t, 1);
+            }
+        }
+        return at;
+    };
+    const auto cols = holders(g.nx, ntx, g.edge[0], g.edge[1], k), rows = holders(g.ny, nty, g.edge[2], g.edge[3], k);
+    std::vector<int> count((size_t)ntx * nty, 0);
+    for (int w = 0; w < g.walls; ++w)
+        for (const auto& b : rows[g.wall[w] / g.nx])
+            for (const auto& a : cols[g.wall[w] % g.nx]) count[(size_t)b.first * ntx + a.first] += a.second * b.second;
+    return *std::max_element(count.begin(), count.end());
+}
+
 }  // namespace
 
 Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmode, int sms)
 {
     Plan best;
     int64_t nodes = 0;
-    bool dirichlet = false, walls = false;
+    bool dirichlet = false;
     for (const GridView& g : grids) {
         nodes += (int64_t)g.nx * g.ny;
         for (int y = 0; y < g.ny; ++y)
@@ -107,7 +128,6 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
     bool dry = false;
     for (const GridView& g : grids) {
         counts.emplace_back(g);
-        walls = walls || counts.back().walls;
         dry = dry || !counts.back().c.empty();
     }
     // without dry nodes to leave out, FP64 gains only where the tile kernel
@@ -157,7 +177,6 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
                 s.hw = (ww + 6) / 2;
                 s.rows = wh + 2;
                 s.ghosts = 2 * (ww + 2) + 2 * wh;
-                s.walls = !f64 && walls ? ww * wh : 0;
                 s.dirs = dirichlet ? 2 * (ww + wh) : 0;
                 const size_t smem = s.cells() * per_cell;
                 if (smem > MAX_SMEM) continue;
@@ -243,6 +262,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
     for (size_t i = 0; i < grids.size(); ++i) {
         const GridView& g = grids[i];
         const int ntx = tiles(g.nx, btw), nty = tiles(g.ny, bth);
+        if (!f64 && g.walls > 0) best.shape.walls = std::max(best.shape.walls, most_walls(g, ntx, nty, best.k));
         for (int b = 0; b < nty; ++b)
             for (int a = 0; a < ntx; ++a) {
                 Item it{(int)i, cut(g.nx, ntx, a), cut(g.nx, ntx, a + 1), cut(g.ny, nty, b), cut(g.ny, nty, b + 1), 0, g.off};

@@ -18,6 +18,7 @@ struct GridView {
     const uint8_t* type;  // host [ny][pitch]
     long long off;        // first element in the packed arrays
     int walls, dirichlet; // nodes with a bounce-back link, Dirichlet nodes
+    const int* wall;      // the former (j * nx + i)
 };
 
 // One step of an FP32 batch, us, of 64 x 16 tiles (one launch of the tile
