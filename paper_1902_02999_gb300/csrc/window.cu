@@ -10,10 +10,6 @@ namespace maclab {
 namespace window {
 namespace {
 
-#ifndef MACLAB_WINDOW_K
-#define MACLAB_WINDOW_K 0  // tuning builds: force the steps per launch
-#endif
-
 constexpr size_t MAX_SMEM = 227 * 1024 - 2048;
 
 // Cost model in SM cycles, fitted to clock readings inside the kernel and to
@@ -39,6 +35,11 @@ double f64_cycles(double nodes, double instructions, double shared)
     return STEP_CYCLES + instructions * std::max(66.0 * std::ceil(warps / 4), 19.0 * warps);
 }
 
+// tiles across an axis of n nodes for tiles of at most t; a tile that does
+// not span the axis has two nodes at least
+int tiles(int n, int t) { return std::max(1, std::min((n + t - 1) / t, std::max(1, n / 2))); }
+int cut(int n, int nt, int i) { return (int)((int64_t)n * i / nt); }
+
 // nodes that are not solid in [0, x) x [0, y), row length nx + 1 (empty when
 // no node is solid)
 struct Counts {
@@ -63,17 +64,31 @@ struct Counts {
             }
         }
     }
+    // tiles that hold a node that is not solid (cx: scratch)
+    int tiles_with_nodes(const GridView& g, int ntx, int nty, std::vector<int>& cx) const
+    {
+        if (c.empty()) return ntx * nty;
+        cx.resize(ntx + 1);
+        for (int a = 0; a <= ntx; ++a) cx[a] = cut(g.nx, ntx, a);
+        int n = 0;
+        for (int b = 0; b < nty; ++b) {
+            const int* r0 = &c[(size_t)cut(g.ny, nty, b) * w];
+            const int* r1 = &c[(size_t)cut(g.ny, nty, b + 1) * w];
+            int before = r1[0] - r0[0];
+            for (int a = 1; a <= ntx; ++a) {
+                const int upto = r1[cx[a]] - r0[cx[a]];
+                n += upto > before;
+                before = upto;
+            }
+        }
+        return n;
+    }
     int operator()(int x0, int x1, int y0, int y1) const
     {
         if (c.empty()) return (x1 - x0) * (y1 - y0);
         return c[(size_t)y1 * w + x1] - c[(size_t)y0 * w + x1] - c[(size_t)y1 * w + x0] + c[(size_t)y0 * w + x0];
     }
 };
-
-// tiles across an axis of n nodes for tiles of at most t; a tile that does
-// not span the axis has two nodes at least
-int tiles(int n, int t) { return std::max(1, std::min((n + t - 1) / t, std::max(1, n / 2))); }
-int cut(int n, int nt, int i) { return (int)((int64_t)n * i / nt); }
 
 // The most nodes with a bounce-back link in the window of any of a grid's nt
 // tiles (nodes that windows wrap onto more than once count each time).
@@ -137,6 +152,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
     static const int TH[] = {2, 4, 8, 12, 16, 24, 32, 48};
     static const int KS[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
     const size_t per_cell = f64 ? cell_bytes<double>() : cell_bytes<float>();
+    std::vector<int> cx;
     double best_cost = 1e300, one_step = 0;
     int btw = 0, bth = 0;
     for (int tw : TW)
@@ -149,10 +165,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
             for (size_t i = 0; i < grids.size(); ++i) {
                 const GridView& g = grids[i];
                 const int ntx = tiles(g.nx, tw), nty = tiles(g.ny, th);
-                for (int b = 0; b < nty; ++b)
-                    for (int a = 0; a < ntx; ++a)
-                        wet += counts[i].c.empty() ||
-                               counts[i](cut(g.nx, ntx, a), cut(g.nx, ntx, a + 1), cut(g.ny, nty, b), cut(g.ny, nty, b + 1)) > 0;
+                wet += counts[i].tiles_with_nodes(g, ntx, nty, cx);
                 mw = std::max(mw, (g.nx + ntx - 1) / ntx);
                 mh = std::max(mh, (g.ny + nty - 1) / nty);
             }
@@ -163,7 +176,7 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
                                      : 2 * STEP_CYCLES + WARP_F32 * mw * mh / 64);
             if (bare >= best_cost) continue;
             for (int k : KS) {
-                if (MACLAB_WINDOW_K > 0 && k != MACLAB_WINDOW_K) continue;
+                if (bare + (LAUNCH_CYCLES + BLOCK_CYCLES) / k >= best_cost) continue;
                 // the largest window over the grids
                 int ww = 0, wh = 0;
                 for (const GridView& g : grids) {
