@@ -371,7 +371,8 @@ int maclab_get_profile(maclab_t sim, double* step_kernel_ms, int64_t* launches);
  * blocks; 5, 6 and 8 are tried on FP32 MacLABSWE handles only, and the
  * temporal block depth is set to the winner's (1 unless 6 or 8 wins).  On a
  * small grid the several-step launches of maclab_step are timed too and kept
- * on when they beat every shape.  Each shape runs 2 + trial_steps steps; the
+ * on when they beat every shape; *choice is then the fastest shape with one step
+ * per launch (not 6 or 8), which calls too short for them take.  Each shape runs 2 + trial_steps steps; the
  * state, step count and time are restored afterwards (results are bitwise
  * identical for every shape).  Allocates and frees a copy of the state.
  * Synchronises. */

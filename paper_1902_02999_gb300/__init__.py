@@ -286,8 +286,10 @@ class Simulation:
     def autotune(self, trial_steps: int = 20) -> int:
         """Pick the fastest step-kernel launch shape for this grid (0 = tile
         kernel, 1..4 = strip kernel with 8/16/32/64 rows, 5 = TMA-staged tile
-        kernel, 6 = tile kernel with two steps per launch on clean tiles);
-        state unchanged."""
+        kernel, 6 = tile kernel with two steps per launch on clean tiles, 7 =
+        row march, 8 = row march with two steps per pass); state unchanged.
+        Where the several-step launches of a small grid beat every shape they
+        stay on, and the shape is the one for calls too short for them."""
         c = ctypes.c_int()
         self._check(self._lib.maclab_autotune(self._h, int(trial_steps), ctypes.byref(c)))
         info = _abi.Info()

@@ -11,6 +11,7 @@
 #include "maclab_march.cuh"
 #include "maclab_elab.cuh"
 #include "window.h"
+#include "autotune.h"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -1502,25 +1503,19 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
     s->kernel_chosen = true;  // time the launch shapes themselves
     const int ty0 = s->ty;
     const int prof0 = s->profiling;
-    // candidates: 0 = tile kernel; k = 1..4 strip kernel with 4 << k rows;
-    // 5 = TMA-staged tile kernel; 6 = tile kernel with two steps per launch
-    // on clean tiles (FP32 MacLABSWE steps only); 7 = row-march kernel;
-    // 8 = row-march kernel with two steps per pass on plain strip blocks
-    // (FP32 MacLABSWE steps only)
     const int rows[5] = {0, 8, 16, 32, 64};
     const bool try_pairs = s->prec == MACLAB_F32 && !s->elab && !s->newlevel;
-    const int ncand = 9;
-    double best = 1e300;
-    int best_k = 0;
+    double took[autotune::CANDIDATES], several = INFINITY;  // of each candidate
+    std::fill(took, took + autotune::CANDIDATES, INFINITY);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     s->profiling = true;  // one launch per step (no graph replay) while timing
     int rc = MACLAB_OK;
     s->tblock = 1;
-    for (int k = 0; k < ncand && rc == MACLAB_OK; ++k) {
+    for (int k = 0; k < autotune::CANDIDATES && rc == MACLAB_OK; ++k) {
         if (k == 5 && !s->tma_ok) continue;
-        if ((k == 6 || k == 8) && !try_pairs) continue;
+        if (autotune::two_steps(k) && !try_pairs) continue;
         if (k == 7) s->tblock = 1;
         if (k == 8) {
             if ((rc = maclab_set_temporal_block(s, 2)) != MACLAB_OK) break;
@@ -1548,13 +1543,9 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
         cudaEventSynchronize(e1);
         float ms = 0;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (rc == MACLAB_OK && ms < best) {
-            best = ms;
-            best_k = k;
-        }
+        if (rc == MACLAB_OK) took[k] = ms;
     }
     // several steps per launch, kept on when it beats every shape
-    bool keep_window = false;
     if (rc == MACLAB_OK && s->wplan.k > 0) {
         s->tblock = 1;
         s->kernel_chosen = false;
@@ -1568,17 +1559,19 @@ int maclab_autotune(maclab_t s, int trial_steps, int* choice)
             cudaEventSynchronize(e1);
             float ms = 0;
             cudaEventElapsedTime(&ms, e0, e1);
-            keep_window = rc == MACLAB_OK && ms < best;
+            if (rc == MACLAB_OK) several = ms;
         }
         s->wplan.min_steps = min_steps;
     }
-    s->kernel_chosen = rc == MACLAB_OK ? !keep_window : chosen0;
+    const autotune::Choice won = autotune::choose(took, several);
+    const int best_k = won.shape;
+    s->kernel_chosen = std::isfinite(several) ? !won.several : chosen0;  // (not tried in the other forms)
     s->events_used = 0;
     s->profiling = prof0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     s->kernel = kernel_of_choice(best_k);
-    s->tblock = !keep_window && (best_k == 6 || best_k == 8) ? 2 : 1;
+    s->tblock = autotune::two_steps(best_k) ? 2 : 1;
     if (best_k >= 1 && best_k <= 4) {
         s->ty = std::min(rows[best_k], s->grid.ny);
     } else {
