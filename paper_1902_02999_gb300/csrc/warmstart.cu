@@ -941,6 +941,7 @@ struct maclab_ws_s {
     bf16* X = nullptr;          // [B][R][R][16]
     std::vector<bf16*> H;       // H_1 .. H_{L+1}, [B][R][R][C]
     std::vector<bf16*> HR;      // relu of each that a layer on tcgen05 reads, stored by the layer that writes it; or nullptr
+    bf16* rectified = nullptr;  // their memory
     int sms = 152;
     bf16* G[2] = {nullptr, nullptr};  // gradient ping-pong [B][R][R][C]
     std::vector<bf16*> GK;      // kept gradients w.r.t. H_1 .. H_{L+1} (maclab_ws_keep_gradients)
@@ -1148,7 +1149,9 @@ void launch_conv(maclab_ws_t w, const ConvArgs& a, int batch)
 {
     const int segs = a.R / CONV_M;
     if (w->cfg.tensor_path == 0 && launch_conv5(w, a, batch)) return;
-    if (w->cfg.tensor_path == 1 && a.Cin % TC_KS == 0 && a.Cout % TC_N == 0 && (a.R * a.R) % TC_M == 0) {
+    // (path 0 without stored rectified copies: the tcgen05 kernel that rectifies as it stages)
+    const bool staged = w->cfg.tensor_path == 1 || (w->cfg.tensor_path == 0 && a.relu_in && !a.XR);
+    if (staged && a.Cin % TC_KS == 0 && a.Cout % TC_N == 0 && (a.R * a.R) % TC_M == 0) {
         dim3 grid(batch * (a.R * a.R / TC_M), a.Cout / TC_N);
         ws_conv_tc_kernel<<<grid, TC_THREADS, TC_SMEM, w->stream>>>(a, w->tc_err);
     } else if (a.Cout % 128 == 0) {
@@ -1406,16 +1409,8 @@ int maclab_ws_create(const maclab_ws_config* cfg, void* stream, maclab_ws_t* out
     for (const auto& L : w->layers) biases += L.cout;
     ok = ok && walloc(w, &w->bpart, BG_BLOCKS * biases) && walloc(w, &w->part, w->part_floats) && walloc(w, &w->dpart, 2 * 1024);
     w->H.assign(w->layers.size() - 1, nullptr);
-    // the tcgen05 path keeps relu(H) beside H (one allocation for both)
-    // where the layer that reads it runs there: every layer, or with channel
-    // counts only the head takes, the last one
-    const bool tc = cfg->tensor_path == 0 && conv5_shape(R, C, IO) && tensor_map_encoder();
+    for (size_t l = 0; ok && l < w->H.size(); ++l) ok = walloc(w, &w->H[l], P * C);
     w->HR.assign(w->H.size(), nullptr);
-    for (size_t l = 0; ok && l < w->H.size(); ++l) {
-        const bool rect = tc && (conv5_shape(R, C, C) || l + 1 == w->H.size());
-        ok = walloc(w, &w->H[l], P * C * (rect ? 2 : 1));
-        if (ok && rect) w->HR[l] = w->H[l] + P * C;
-    }
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev);
     ok = ok && walloc(w, &w->Wf_all, w->nparam) && walloc(w, &w->Wb_all, w->nparam);
@@ -1433,6 +1428,15 @@ int maclab_ws_create(const maclab_ws_config* cfg, void* stream, maclab_ws_t* out
     if (!ok) {
         maclab_ws_destroy(w);
         return wfail(nullptr, MACLAB_E_NOMEM, "warm-start device allocation failed");
+    }
+    // the tcgen05 path keeps relu(H) besides H where the layer that reads it
+    // runs there: every layer, or with channel counts only the head takes, the
+    // last one.  Without memory for them those layers take the kernels that
+    // rectify as they stage.
+    if (cfg->tensor_path == 0 && conv5_shape(R, C, IO) && tensor_map_encoder()) {
+        const size_t first = conv5_shape(R, C, C) ? 0 : w->H.size() - 1;
+        if (walloc(w, &w->rectified, (w->H.size() - first) * P * C))
+            for (size_t l = first; l < w->H.size(); ++l) w->HR[l] = w->rectified + (l - first) * P * C;
     }
     // initial weights: normal(0, sqrt(2 / fan_in)) by Box-Muller on SplitMix64;
     // the residual branches start small and the head at zero
@@ -1557,8 +1561,18 @@ int maclab_ws_keep_gradients(maclab_ws_t w, int on)
     if (on && w->GK.empty()) {
         const size_t P = (size_t)w->cfg.max_batch * w->cfg.res * w->cfg.res;
         std::vector<bf16*> k(w->H.size(), nullptr);
-        for (auto& p : k)
+        for (auto& p : k) {
+            if (walloc(w, &p, P * w->cfg.channels)) continue;
+            // the rectified copies make room
+            if (!w->rectified) return wfail(w, MACLAB_E_NOMEM, "keep_gradients: out of memory");
+            const cudaError_t e = cudaStreamSynchronize(w->stream);
+            if (e != cudaSuccess) return wfail(w, MACLAB_E_CUDA, std::string("keep_gradients: ") + cudaGetErrorString(e));
+            w->bufs.erase(std::find(w->bufs.begin(), w->bufs.end(), (void*)w->rectified));
+            cudaFree(w->rectified);
+            w->rectified = nullptr;
+            std::fill(w->HR.begin(), w->HR.end(), nullptr);
             if (!walloc(w, &p, P * w->cfg.channels)) return wfail(w, MACLAB_E_NOMEM, "keep_gradients: out of memory");
+        }
         w->GK = k;
     }
     w->keep = on != 0;
