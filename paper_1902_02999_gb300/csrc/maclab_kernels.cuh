@@ -305,14 +305,11 @@ __device__ __forceinline__ Bed64 bed_at(const Fields<double>& f, size_t i, doubl
     return bed_of(d1, d2, d3, d4, d5, d6, d7, d8);
 }
 
-// Source-side quantities of one node (see the header comment).
-template <typename T, int FM>
-__device__ __forceinline__ void derive(const Coef<T>& c, const Raw<T>& r, Src<T>& s)
+// Source-side quantities of one node in FP32 (see the header comment).
+template <int FM>
+__device__ __forceinline__ void derive32(const Coef<float>& c, const Raw<float>& r, Src<float>& s)
 {
-    if constexpr (std::is_same<T, double>::value) {
-        derive64<FM>(c, r, s);
-        return;
-    }
+    using T = float;
     using O = Op<T>;
     T u = r.u, v = r.v, wfx = c.wfx, wfy = c.wfy, Om = c.Om;
     if (r.flip) {  // specular ghost: normal components reversed, rotation sense too
@@ -367,6 +364,15 @@ __device__ __forceinline__ void derive(const Coef<T>& c, const Raw<T>& r, Src<T>
     s.o4 = O::sub(dm, t4);
     s.eta = eta;
     s.D = D;
+}
+
+template <typename T, int FM>
+__device__ __forceinline__ void derive(const Coef<T>& c, const Raw<T>& r, Src<T>& s)
+{
+    if constexpr (std::is_same<T, double>::value)
+        derive64<FM>(c, r, s);
+    else
+        derive32<FM>(c, r, s);
 }
 
 // Source quantities of two nodes at once (FP32): the operations of derive,
@@ -462,69 +468,51 @@ __device__ __forceinline__ void derive2(const Coef2& c, const Raw<float>& r0, co
     s.D = D;
 }
 
-// New eta, u, v of a node from its streamed sums (Sh, Sx, Sy: the first
+// New eta, u, v of a node in FP32 from its streamed sums (Sh, Sx, Sy: the first
 // terms of Eqs. Mac.lb.6 / Mac.lb.7 over the eight incoming outgoing values)
 // and the (eta, D) of its eight neighbours (m: row above, c: same row,
 // p: row below; L / C / R: column left / same / right), in the perturbation
 // form; eta, D, ownh, hFx, hFy are the node's own source quantities.  Every
-// kernel that updates fast-path nodes ends in this one function, so their
-// results agree bitwise.
-template <typename T, typename V2 = typename Vec2<T>::type>
-__device__ __forceinline__ void update_tail(const Coef<T>& K, T Sh, T Sx, T Sy, V2 mL, V2 mC, V2 mR, V2 cL, V2 cR,
-                                            V2 pL, V2 pC, V2 pR, T eta, T D, T ownh, T hFx, T hFy, bool noslip,
-                                            T& oe, T& ou, T& ov)
+// FP32 kernel that updates fast-path nodes takes these operations in this
+// order (the row march two nodes at a time, gather_pair), so their results
+// agree bitwise; FP64 ends in update64.
+__device__ __forceinline__ void update_tail(const Coef<float>& K, float Sh, float Sx, float Sy, float2 mL, float2 mC,
+                                            float2 mR, float2 cL, float2 cR, float2 pL, float2 pC, float2 pR, float eta,
+                                            float D, float ownh, float hFx, float hFy, bool noslip, float& oe, float& ou,
+                                            float& ov)
 {
-    using O = Op<T>;
-    const T q = T(0.25);
-    // lambda-weighted stencils of eta (.x) and D (.y): sum, x-moment, y-moment
-    T Se, Sd, Xe, Xd, Ye, Yd;
-#ifndef MACLAB_SCALAR_STENCIL
-    if constexpr (std::is_same<T, float>::value) {
-        // eta and D take the same operations: the two lanes of one paired
-        // instruction (each lane rounded as the scalar operation)
-        using P = Op2;
-        const float2 q2 = splat(q);
-        const float2 ML = P::fma(q2, P::add(mL, pL), cL), MR = P::fma(q2, P::add(mR, pR), cR);
-        const float2 S = P::add(P::add(ML, MR), P::add(mC, pC));
-        const float2 X = P::sub(ML, MR);
-        const float2 Y = P::fma(q2, P::sub(P::add(mL, mR), P::add(pL, pR)), P::sub(mC, pC));
-        Se = S.x, Sd = S.y, Xe = X.x, Xd = X.y, Ye = Y.x, Yd = Y.y;
-    } else
-#endif
-    {
-        const T MLe = O::fma(q, O::add(mL.x, pL.x), cL.x);
-        const T MRe = O::fma(q, O::add(mR.x, pR.x), cR.x);
-        const T MLd = O::fma(q, O::add(mL.y, pL.y), cL.y);
-        const T MRd = O::fma(q, O::add(mR.y, pR.y), cR.y);
-        Se = O::add(O::add(MLe, MRe), O::add(mC.x, pC.x));
-        Sd = O::add(O::add(MLd, MRd), O::add(mC.y, pC.y));
-        Xe = O::sub(MLe, MRe), Xd = O::sub(MLd, MRd);
-        Ye = O::fma(q, O::sub(O::add(mL.x, mR.x), O::add(pL.x, pR.x)), O::sub(mC.x, pC.x));
-        Yd = O::fma(q, O::sub(O::add(mL.y, mR.y), O::add(pL.y, pR.y)), O::sub(mC.y, pC.y));
-    }
-    const T A = O::mul(K.G6, D), B = O::mul(K.G6, eta);
+    using O = Op<float>;
+    using P = Op2;
+    // lambda-weighted stencils of eta (.x) and D (.y): sum, x-moment,
+    // y-moment.  Both take the same operations: the two lanes of one paired
+    // instruction (each lane rounded as the scalar operation).
+    const float2 q2 = splat(0.25f);
+    const float2 ML = P::fma(q2, P::add(mL, pL), cL), MR = P::fma(q2, P::add(mR, pR), cR);
+    const float2 S = P::add(P::add(ML, MR), P::add(mC, pC));
+    const float2 X = P::sub(ML, MR);
+    const float2 Y = P::fma(q2, P::sub(P::add(mL, mR), P::add(pL, pR)), P::sub(mC, pC));
+    const float A = O::mul(K.G6, D), B = O::mul(K.G6, eta);
     // ownh already holds the receiver-only bed part 5 G6 eta_x D_x
-    const T eta1 = O::add(O::add(ownh, Sh), O::fma(A, Se, O::mul(-B, Sd)));
-    const T hu1 = O::fma(K.e, O::add(Sx, O::fma(A, Xe, O::mul(-B, Xd))), hFx);
-    const T hv1 = O::fma(K.e, O::add(Sy, O::fma(A, Ye, O::mul(-B, Yd))), hFy);
-    const T inv = O::rcp(O::add(D, eta1));
+    const float eta1 = O::add(O::add(ownh, Sh), O::fma(A, S.x, O::mul(-B, S.y)));
+    const float hu1 = O::fma(K.e, O::add(Sx, O::fma(A, X.x, O::mul(-B, X.y))), hFx);
+    const float hv1 = O::fma(K.e, O::add(Sy, O::fma(A, Y.x, O::mul(-B, Y.y))), hFy);
+    const float inv = O::rcp(O::add(D, eta1));
     oe = eta1;
-    ou = noslip ? T(0) : O::mul(hu1, inv);
-    ov = noslip ? T(0) : O::mul(hv1, inv);
+    ou = noslip ? 0.f : O::mul(hu1, inv);
+    ov = noslip ? 0.f : O::mul(hv1, inv);
 }
 
-// Streamed sums of the first terms of Eqs. Mac.lb.6 / Mac.lb.7 from the
+// Streamed sums of the first terms of Eqs. Mac.lb.6 / Mac.lb.7 (FP32) from the
 // eight incoming values, grouped as (left column), (right column), centre:
 // a1 = cL_o1 + mL_o2 and a2 = cR_o5 + mR_o4 and sym = mL_o2 + mR_o4 + mC_o3
 // take only the node's own row and the row above, so a kernel that walks
 // down the rows can form them before the row below exists.
-template <typename T>
-__device__ __forceinline__ void streamed_sums(T a1, T a2, T sym, T mC_o3, T pL_o8, T pR_o6, T pC_o7, T& Sh, T& Sx,
-                                              T& Sy)
+__device__ __forceinline__ void streamed_sums(float a1, float a2, float sym, float mC_o3, float pL_o8, float pR_o6,
+                                              float pC_o7, float& Sh, float& Sx, float& Sy)
 {
-    using O = Op<T>;
-    const T OL = O::add(a1, pL_o8);
-    const T OR = O::add(a2, pR_o6);
+    using O = Op<float>;
+    const float OL = O::add(a1, pL_o8);
+    const float OR = O::add(a2, pR_o6);
     Sh = O::add(O::add(OL, OR), O::add(mC_o3, pC_o7));
     Sx = O::sub(OL, OR);
     Sy = O::sub(sym, O::add(O::add(pL_o8, pR_o6), pC_o7));
@@ -765,9 +753,9 @@ __device__ __forceinline__ void emit_row(const Fields<T>& f, int j, int xl, int 
             using V2 = typename Vec2<T>::type;
             auto ed = [](const Src<T>& q) { return V2{q.eta, q.D}; };
             T Sh, Sx, Sy;
-            streamed_sums<T>(O::add(cL.o1, mL.o2), O::add(cR.o5, mR.o4), O::add(O::add(mL.o2, mR.o4), mC.o3), mC.o3,
+            streamed_sums(O::add(cL.o1, mL.o2), O::add(cR.o5, mR.o4), O::add(O::add(mL.o2, mR.o4), mC.o3), mC.o3,
                              pL.o8, pR.o6, pC.o7, Sh, Sx, Sy);
-            update_tail<T>(K, Sh, Sx, Sy, ed(mL), ed(mC), ed(mR), ed(cL), ed(cR), ed(pL), ed(pC), ed(pR), cC.eta, cC.D,
+            update_tail(K, Sh, Sx, Sy, ed(mL), ed(mC), ed(mR), ed(cL), ed(cR), ed(pL), ed(pC), ed(pR), cC.eta, cC.D,
                            cC.ownh, cC.hFx, cC.hFy, noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
         }
     }
@@ -1375,18 +1363,18 @@ __device__ __forceinline__ void node_update(const DR& sm, int lr, int lc, const 
                  Eta8{sm.ed(lr - 1, lc - 1).x, sm.ed(lr - 1, lc).x, sm.ed(lr - 1, lc + 1).x, sm.ed(lr, lc - 1).x,
                       sm.ed(lr, lc + 1).x, sm.ed(lr + 1, lc - 1).x, sm.ed(lr + 1, lc).x, sm.ed(lr + 1, lc + 1).x},
                  eta, D, ownh, hFx, hFy, bd, noslip, oe, ou, ov);
-        return;
+    } else {
+        using O = Op<T>;
+        const T cL_o1 = sm.o(0, lr, lc - 1), mL_o2 = sm.o(1, lr - 1, lc - 1), pL_o8 = sm.o(7, lr + 1, lc - 1);
+        const T cR_o5 = sm.o(4, lr, lc + 1), mR_o4 = sm.o(3, lr - 1, lc + 1), pR_o6 = sm.o(5, lr + 1, lc + 1);
+        const T mC_o3 = sm.o(2, lr - 1, lc), pC_o7 = sm.o(6, lr + 1, lc);
+        T Sh, Sx, Sy;
+        streamed_sums(O::add(cL_o1, mL_o2), O::add(cR_o5, mR_o4), O::add(O::add(mL_o2, mR_o4), mC_o3), mC_o3, pL_o8,
+                         pR_o6, pC_o7, Sh, Sx, Sy);
+        update_tail(K, Sh, Sx, Sy, sm.ed(lr - 1, lc - 1), sm.ed(lr - 1, lc), sm.ed(lr - 1, lc + 1), sm.ed(lr, lc - 1),
+                       sm.ed(lr, lc + 1), sm.ed(lr + 1, lc - 1), sm.ed(lr + 1, lc), sm.ed(lr + 1, lc + 1), eta, D, ownh,
+                       hFx, hFy, noslip, oe, ou, ov);
     }
-    using O = Op<T>;
-    const T cL_o1 = sm.o(0, lr, lc - 1), mL_o2 = sm.o(1, lr - 1, lc - 1), pL_o8 = sm.o(7, lr + 1, lc - 1);
-    const T cR_o5 = sm.o(4, lr, lc + 1), mR_o4 = sm.o(3, lr - 1, lc + 1), pR_o6 = sm.o(5, lr + 1, lc + 1);
-    const T mC_o3 = sm.o(2, lr - 1, lc), pC_o7 = sm.o(6, lr + 1, lc);
-    T Sh, Sx, Sy;
-    streamed_sums<T>(O::add(cL_o1, mL_o2), O::add(cR_o5, mR_o4), O::add(O::add(mL_o2, mR_o4), mC_o3), mC_o3, pL_o8,
-                     pR_o6, pC_o7, Sh, Sx, Sy);
-    update_tail<T>(K, Sh, Sx, Sy, sm.ed(lr - 1, lc - 1), sm.ed(lr - 1, lc), sm.ed(lr - 1, lc + 1), sm.ed(lr, lc - 1),
-                   sm.ed(lr, lc + 1), sm.ed(lr + 1, lc - 1), sm.ed(lr + 1, lc), sm.ed(lr + 1, lc + 1), eta, D, ownh,
-                   hFx, hFy, noslip, oe, ou, ov);
 }
 
 // Phases B and C of a tile whose phase A is complete and visible; `tile`

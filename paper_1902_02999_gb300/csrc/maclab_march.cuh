@@ -712,11 +712,8 @@ struct BatchGeom {
 };
 }  // namespace march
 
-#ifndef MACLAB_MARCH_BATCH_MINB
-#define MACLAB_MARCH_BATCH_MINB 5
-#endif
 template <int FM>
-__global__ void __launch_bounds__(march::THREADS, MACLAB_MARCH_BATCH_MINB)
+__global__ void __launch_bounds__(march::THREADS, 5)
 step_march_batch_kernel(const __grid_constant__ Fields<float> bases, const BatchInst<float>* __restrict__ insts,
                         const uint8_t* __restrict__ active, const __grid_constant__ march::BatchGeom g, int parity)
 {
