@@ -143,10 +143,9 @@ template <> struct Op<double> {
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-    // CUDA's correctly rounded reciprocal and root.  (The hardware's
-    // approximations and a third-order step each took 5 % less time, 388
-    // against 409 us a step on 2999 x 701 nodes, with a root up to 0.755 ulp
-    // off.)
+    // CUDA's correctly rounded reciprocal and root.  (Both from hardware
+    // approximations and one third-order step: 388 against 409 us a step on
+    // 2999 x 701 nodes, but roots up to 0.755 ulp off.)
     static __device__ __forceinline__ double rcp(double a) { return 1.0 / a; }
     static __device__ __forceinline__ double sqrt(double a) { return ::sqrt(a); }
 };
@@ -753,10 +752,10 @@ __device__ __forceinline__ void emit_row(const Fields<T>& f, int j, int xl, int 
             using V2 = typename Vec2<T>::type;
             auto ed = [](const Src<T>& q) { return V2{q.eta, q.D}; };
             T Sh, Sx, Sy;
-            streamed_sums(O::add(cL.o1, mL.o2), O::add(cR.o5, mR.o4), O::add(O::add(mL.o2, mR.o4), mC.o3), mC.o3,
-                             pL.o8, pR.o6, pC.o7, Sh, Sx, Sy);
+            streamed_sums(O::add(cL.o1, mL.o2), O::add(cR.o5, mR.o4), O::add(O::add(mL.o2, mR.o4), mC.o3), mC.o3, pL.o8,
+                          pR.o6, pC.o7, Sh, Sx, Sy);
             update_tail(K, Sh, Sx, Sy, ed(mL), ed(mC), ed(mR), ed(cL), ed(cR), ed(pL), ed(pC), ed(pR), cC.eta, cC.D,
-                           cC.ownh, cC.hFx, cC.hFy, noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
+                        cC.ownh, cC.hFx, cC.hFy, noslip, oe[k - 1], ou[k - 1], ov[k - 1]);
         }
     }
     if (j >= f.ny || okmask == 0) return;
@@ -1370,10 +1369,10 @@ __device__ __forceinline__ void node_update(const DR& sm, int lr, int lc, const 
         const T mC_o3 = sm.o(2, lr - 1, lc), pC_o7 = sm.o(6, lr + 1, lc);
         T Sh, Sx, Sy;
         streamed_sums(O::add(cL_o1, mL_o2), O::add(cR_o5, mR_o4), O::add(O::add(mL_o2, mR_o4), mC_o3), mC_o3, pL_o8,
-                         pR_o6, pC_o7, Sh, Sx, Sy);
+                      pR_o6, pC_o7, Sh, Sx, Sy);
         update_tail(K, Sh, Sx, Sy, sm.ed(lr - 1, lc - 1), sm.ed(lr - 1, lc), sm.ed(lr - 1, lc + 1), sm.ed(lr, lc - 1),
-                       sm.ed(lr, lc + 1), sm.ed(lr + 1, lc - 1), sm.ed(lr + 1, lc), sm.ed(lr + 1, lc + 1), eta, D, ownh,
-                       hFx, hFy, noslip, oe, ou, ov);
+                    sm.ed(lr, lc + 1), sm.ed(lr + 1, lc - 1), sm.ed(lr + 1, lc), sm.ed(lr + 1, lc + 1), eta, D, ownh, hFx,
+                    hFy, noslip, oe, ou, ov);
     }
 }
 
