@@ -173,7 +173,10 @@ typedef struct {
  *   alloc  : optional allocator, NULL for cudaMalloc.
  *   stream : cudaStream_t the handle launches on (NULL = legacy stream).
  * Errors: MACLAB_E_ARG for bad sizes, codes, unpaired periodic edges or
- * misplaced Dirichlet nodes; MACLAB_E_NOMEM; MACLAB_E_CUDA.
+ * misplaced Dirichlet nodes; MACLAB_E_NOMEM; MACLAB_E_CUDA.  Memory that only
+ * makes steps faster (lists and scratch state of several-step launches, FP64
+ * stencils of the still-water depth) is held where it fits beside a marked
+ * state (maclab_mark) and otherwise left out.
  * Uses the current CUDA device. */
 int maclab_create(const maclab_grid* grid, const maclab_params* params, const maclab_bc* bc,
                   const double* zb, const uint8_t* mask, const double* h0, const double* u0,
@@ -320,6 +323,9 @@ int maclab_set_step_kernel(maclab_t sim, int kernel);
  * no-slip or Dirichlet nodes, or for tau <= 0.5.  maclab_set_state restarts
  * the distributions at the equilibrium of the new state.  Per node and step
  * the FP32 form reads 41 bytes and writes 48 (MacLABSWE: 17 and 12).
+ * Where the distributions do not fit, the handle gives up the memory that only
+ * makes MacLABSWE steps faster (see maclab_create): a graph that the caller
+ * captured from this handle before is not valid any more.
  * Synchronises. */
 int maclab_set_relaxation(maclab_t sim, double tau);
 
@@ -352,13 +358,14 @@ int maclab_set_hbar_level(maclab_t sim, int level);
  * MACLAB_E_ARG for k outside 1..2 or k = 2 on an FP64 handle. */
 int maclab_set_temporal_block(maclab_t sim, int k);
 
-/* Kernel timing for benchmarks.  While enabled (on != 0), every step
- * records a CUDA event pair around the launch of the fused step kernel on
- * the handle's stream.  maclab_get_profile synchronises, adds up the
+/* Kernel timing for benchmarks.  While enabled (on != 0), every
+ * launch of a step kernel is recorded by a CUDA event pair around it on the
+ * handle's stream.  maclab_get_profile synchronises, adds up the
  * recorded durations (milliseconds) and the number of steps those launches
  * advanced since profiling was enabled, and clears the record.  Enabling
- * resets it.  With temporal blocking a two-step launch and its companion
- * single-step launches are timed as one record of two steps. */
+ * resets it.  A several-step launch (small grids) is one record of its steps;
+ * with temporal blocking a two-step launch and its companion single-step
+ * launches are timed as one record of two steps. */
 int maclab_set_profiling(maclab_t sim, int on);
 int maclab_get_profile(maclab_t sim, double* step_kernel_ms, int64_t* launches);
 

@@ -93,7 +93,9 @@ int maclab_ws_train_step(maclab_ws_t ws, int batch, int out_ch, const float* x_d
  * maclab_ws_gradients / maclab_ws_train_step leaves the loss gradient with
  * respect to every H_l in a buffer of its own (L + 1 more activation-sized
  * bf16 buffers, allocated on the first call with on = 1 and kept until
- * destroy) instead of overwriting two.  MACLAB_E_NOMEM if they do not fit. */
+ * destroy) instead of overwriting two.  Where they do not fit beside the
+ * stored rectified activations of tensor_path 0 those are given up (the layers
+ * then rectify as they stage); MACLAB_E_NOMEM if they do not fit at all. */
 int maclab_ws_keep_gradients(maclab_ws_t ws, int on);
 
 /* Float copy into out_dev of a tensor the handle stores, as of the last

@@ -39,9 +39,9 @@
 //
 // Measured per step, single-step launches (graph replay where the boundary
 // is steady) -> this kernel: 256 x 256 lake FP32 11.4 -> 1.9 us, 1001 x 333
-// channel FP32 10.1 -> 5.5 us, 400 x 3 tidal strip FP64 49 -> 3.3 us, eight
-// 256 x 256 lakes FP64 195 -> 60 us (148 with the tile kernel's present
-// arithmetic).  Computing the lists' content in every launch instead took
+// channel FP32 10.1 -> 5.5 us, 400 x 3 tidal strip FP64 49 -> 3.4 us, eight
+// 256 x 256 lakes FP64 195 -> 63 us (both with FP64's cheaper arithmetic of
+// today in the second figure).  Computing the lists' content in every launch instead took
 // 3.3, 9.0, 5.4 and 70 us.  Inside a launch (clock readings, 40 x 24 tile,
 // k = 6, 910 pairs): loads 2,000 cycles, a step 1,700 (A) + 2,100 (B), store
 // 1,300; the FP32 pipe is busy about half of a step.
