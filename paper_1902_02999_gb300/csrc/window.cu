@@ -4,7 +4,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <utility>
 
 namespace maclab {
 namespace window {
@@ -94,24 +93,34 @@ struct Counts {
 // tiles (nodes that windows wrap onto more than once count each time).
 int most_walls(const GridView& g, int ntx, int nty, int k)
 {
-    // per column and row: the tiles whose windows hold it, and how often
-    auto holders = [](int n, int nt, int lo_kind, int hi_kind, int halo) {
-        std::vector<std::vector<std::pair<int, int>>> at(n);
-        for (int t = 0; t < nt; ++t) {
-            const Axis a = make_axis(cut(n, nt, t), cut(n, nt, t + 1), n, lo_kind, hi_kind, halo, 1);
-            for (int i = 0; i < a.n; ++i) {
-                auto& q = at[wrapped(a.lo + i, n)];
-                if (!q.empty() && q.back().first == t) ++q.back().second;
-                else q.emplace_back(t, 1);
+    // per column and row: the tiles whose windows hold it (once per hold)
+    struct Holders {
+        std::vector<int> start, tile;
+        Holders(int n, int nt, int lo_kind, int hi_kind, int halo) : start(n + 2, 0)
+        {
+            for (int pass = 0; pass < 2; ++pass) {
+                for (int t = 0; t < nt; ++t) {
+                    const Axis a = make_axis(cut(n, nt, t), cut(n, nt, t + 1), n, lo_kind, hi_kind, halo, 1);
+                    int x = wrapped(a.lo, n);
+                    for (int i = 0; i < a.n; ++i, x = x + 1 == n ? 0 : x + 1) {
+                        if (pass == 0) ++start[x + 2];
+                        else tile[start[x + 1]++] = t;
+                    }
+                }
+                if (pass == 0) {
+                    for (int x = 0; x < n; ++x) start[x + 2] += start[x + 1];
+                    tile.resize(start[n + 1]);
+                }
             }
         }
-        return at;
     };
-    const auto cols = holders(g.nx, ntx, g.edge[0], g.edge[1], k), rows = holders(g.ny, nty, g.edge[2], g.edge[3], k);
+    const Holders cols(g.nx, ntx, g.edge[0], g.edge[1], k), rows(g.ny, nty, g.edge[2], g.edge[3], k);
     std::vector<int> count((size_t)ntx * nty, 0);
-    for (int w = 0; w < g.walls; ++w)
-        for (const auto& b : rows[g.wall[w] / g.nx])
-            for (const auto& a : cols[g.wall[w] % g.nx]) count[(size_t)b.first * ntx + a.first] += a.second * b.second;
+    for (int w = 0; w < g.walls; ++w) {
+        const int y = g.wall[w] / g.nx, x = g.wall[w] - y * g.nx;
+        for (int j = rows.start[y]; j < rows.start[y + 1]; ++j)
+            for (int i = cols.start[x]; i < cols.start[x + 1]; ++i) ++count[(size_t)rows.tile[j] * ntx + cols.tile[i]];
+    }
     return *std::max_element(count.begin(), count.end());
 }
 
@@ -210,9 +219,13 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
                 const int fit = std::max(1, std::min((int)(MAX_SMEM / smem), 65536 / (128 * threads)));
                 const int64_t per_sm = (wet + sms - 1) / sms;
                 const double waves = (double)((per_sm + fit - 1) / fit), shared = (double)std::min<int64_t>(per_sm, fit);
+                // with several blocks on an SM one block's loads hide behind another's steps
+                auto whole = [&](double c) {
+                    return LAUNCH_CYCLES + (fit > 1 ? BLOCK_CYCLES + waves * c : waves * (BLOCK_CYCLES + c));
+                };
                 double cyc = LOAD_CELL * ww * wh * shared, first = 0;  // first: with the last step alone
                 const double ghosts = (mw >= ww ? 2.0 * wh : 0) + (mh >= wh ? 2.0 * ww : 0);
-                for (int m = k; m >= 1; --m) {
+                for (int m = k; m >= 1 && whole(cyc) < best_cost * k; --m) {
                     // nodes derived and updated with m steps to take
                     const double da = std::min(ww, mw + 2 * m) * (double)std::min(wh, mh + 2 * m);
                     const double db = std::min(ww, mw + 2 * m - 2) * (double)std::min(wh, mh + 2 * m - 2);
@@ -221,10 +234,6 @@ Plan make_plan(const std::vector<GridView>& grids, bool batch, bool f64, int fmo
                     if (m == 1) first = LOAD_CELL * ww * wh * shared + step;
                     cyc += step;
                 }
-                // with several blocks on an SM one block's loads hide behind another's steps
-                auto whole = [&](double c) {
-                    return LAUNCH_CYCLES + (fit > 1 ? BLOCK_CYCLES + waves * c : waves * (BLOCK_CYCLES + c));
-                };
                 const double cost = whole(cyc) / k;
                 if (cost < best_cost) {
                     best_cost = cost;
