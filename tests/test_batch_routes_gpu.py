@@ -38,6 +38,11 @@ def rows_apart():
     return steady(inputs.random_case(97, 17, 11, edges=(SPECULAR,) * 4, dirichlet_sn=True))
 
 
+def rows_together():
+    """Rows of Dirichlet nodes in one strip block with their inward rows."""
+    return steady(inputs.random_case(97, 51, 11, edges=(SPECULAR,) * 4, dirichlet_sn=True))
+
+
 def walled():
     """Dirichlet nodes whose inward node has a bounce-back link."""
     return steady(inputs.random_case(70, 40, 3, edges=(BOUNCEBACK,) * 4))
@@ -45,6 +50,7 @@ def walled():
 
 BATCHES = {
     "march": (lambda: odd() + lakes(12), "step_march_batch_kernel"),
+    "rows_together": (lambda: odd() + [rows_together()] + lakes(12), "step_march_batch_kernel"),
     "rows_apart": (lambda: odd() + [rows_apart()] + lakes(12), "step_batch_kernel"),
     "walled": (lambda: odd() + [walled()] + lakes(12), "step_batch_kernel"),
     "narrow": (lambda: odd() + [inputs.random_case(64, 64, 1 + i % 2, edges=(SPECULAR,) * 4, solids=False, dirichlet=False)

@@ -35,7 +35,7 @@ def test_bytes(make):
     (12, 12, (BOUNCEBACK,) * 4),
 ])
 def test_walls_everywhere(nx, ny, edges):
-    """Checkerboards of solid nodes: nearly every node has such a link."""
+    """Solid nodes on a lattice: nearly every node has such a link."""
     from paper_1902_02999_gb300 import Batch, Simulation
     case = inputs.random_case(nx, ny, 7, edges=edges, solids=False, dirichlet=False)
     yy, xx = np.mgrid[0:ny, 0:nx]
